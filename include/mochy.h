@@ -65,11 +65,15 @@ typedef struct {
   int64_t hbm_budget_bytes; /* device bytes the context may hold; 0 = no cap */
   int32_t device;           /* CUDA device ordinal; 0 */
   void* stream;             /* cudaStream_t to run on; NULL = own stream */
-  int32_t exact_kernel;     /* mochy_count_exact: 0 = split (open pairs counted
-                               per centre, closed ones enumerated), 1 = plain
-                               per-hyperwedge scan; both give the same counts */
-  int32_t dense_threshold;  /* split kernel: line degree from which a row is
-                               kept as a bitmap; 0 = chosen by the tuner */
+  int32_t exact_kernel;     /* mochy_count_exact: 0 = open pairs counted per
+                               centre, closed ones by levels of overlap (theta
+                               up to 4), else by the split kernels (closed ones
+                               enumerated; see dense_threshold), 1 = plain
+                               per-hyperwedge scan; all give the same counts */
+  int32_t dense_threshold;  /* split kernels: line degree from which a row is
+                               kept as a bitmap; 0 = chosen by the tuner.  A
+                               positive value, or a rest_path, makes exact
+                               counts take the split kernels */
   int32_t rest_path;        /* split kernel, closed candidates of dense rows
                                outside the popcounted combinations: 1 = each
                                lane classifies those of its own word, 2 = they
@@ -451,7 +455,8 @@ void* mochy_stream(mochy_ctx* ctx);
 /* Tracing of the exact count: level 1 records the duration of each of its
  * phases (CUDA events on the context's stream, no effect on the kernels);
  * level 2 also counts kernel statistics (scanned words, candidates, cycles
- * per section), which slows the kernels; 0 turns tracing off.
+ * per section) of the split kernels, which then make the count and are slowed
+ * by it; 0 turns tracing off.
  * mochy_trace_read writes the last traced call as one JSON object into buf
  * (len bytes).  The environment variable MOCHY_TRACE=1 selects level 2 for
  * every context and also prints to stderr. */

@@ -118,6 +118,7 @@ static size_t graph_bytes(const mochy_ctx* c, int which) {
 void release_projection(mochy_ctx* ctx) {
   const int64_t E = ctx->n_edges;
   release_split(ctx);
+  release_levels(ctx);
   if (ctx->nadj || ctx->noff) cudaStreamSynchronize(ctx->stream);
   if (ctx->nadj) {
     int64_t total = 2 * ctx->n_wedges;
@@ -225,6 +226,7 @@ int mochy_create(mochy_ctx** out, const mochy_config* cfg_in) {
   ctx->exact_kernel = cfg.exact_kernel;
   ctx->dense_thr = cfg.dense_threshold;
   ctx->rest_path = cfg.rest_path;
+  ctx->split_forced = cfg.dense_threshold > 0 || cfg.rest_path > 0;
   memset(ctx->last_stats, 0, sizeof(ctx->last_stats));
   int rc = MOCHY_OK;
   auto bail = [&](int code) {
@@ -718,7 +720,7 @@ static int new_like(mochy_ctx* src, mochy_ctx** out) {
   cfg.hbm_budget_bytes = src->budget;
   cfg.stream = src->own_stream ? nullptr : (void*)src->stream;
   cfg.exact_kernel = src->exact_kernel;
-  cfg.dense_threshold = src->dense_thr;
+  cfg.dense_threshold = src->split_forced ? src->dense_thr : 0;
   cfg.rest_path = src->rest_path;
   return mochy_create(out, &cfg);
 }
@@ -832,7 +834,8 @@ int mochy_trace_read(mochy_ctx* ctx, char* buf, int64_t len) {
            "\"heavy_bitmaps\": %llu, \"slots_evicted\": %llu, \"slots_flushed_full\": %llu, "
            "\"dense_rows_counted\": %llu, \"otf_candidates\": %llu, \"otf_words\": %llu, "
            "\"otf_list_entries\": %llu, \"otf_exact\": %llu, \"otf_bitmaps\": %lld}",
-           (long long)ctx->n_dense, ctx->dense_thr_used, (long long)ctx->wwords,
+           (long long)ctx->n_dense, ctx->split_ready ? ctx->dense_thr_used : ctx->dense_thr,
+           (long long)ctx->wwords,
            (long long)ctx->n_heavy, st[0], st[1], st[2], st[3], st[4], st[5], st[6], st[7], st[8],
            st[9], st[10], st[11], st[12], st[13], st[14], st[16], st[17], st[18], st[19],
            st[20], st[21], st[22], (long long)ctx->otf_bitmaps);

@@ -273,7 +273,8 @@ int run_wave(const mochy_config& cfg, const Inputs& in, int g0, int g1, int R, O
   // 4. the union's line graph and split structures
   MOCHY_TRY(project_graph(cx));
   cudaEventRecord(ev.e[2], cx->stream);
-  MOCHY_TRY(prepare_split(cx));
+  bool by_levels;
+  MOCHY_TRY(prepare_exact(cx, &by_levels));
   cudaEventRecord(ev.e[3], cx->stream);
   // 5. one graph launch counts every unit
   const size_t b_hist = (size_t)U * 432 * 8;

@@ -76,6 +76,10 @@ struct SegInfo {
   int64_t dbase, dboff, hbase, nboff, wlo, wn;
 };
 
+constexpr int kMaxPhases = 16;   // traced phases of one count
+
+struct Levels;   // structures of the exact count by levels (levels.cu)
+
 // Scratch arena: grows on demand, freed with the context.
 struct Buffer {
   void* p = nullptr;
@@ -154,6 +158,10 @@ struct mochy_ctx {
   int64_t* d_dbase = nullptr;          // [n_units+1] first dense index per unit
   int64_t wmax = 0;                    // widest unit window, words
 
+  // exact count by levels (built on first use, released with the line graph)
+  mochy::Levels* levels = nullptr;
+  bool split_forced = false;     // the configuration asks for the split kernels
+
   // MoCHy-A+ without the line graph (built on first use after a load):
   // membership bitmaps of the most popular nodes, size planes, and the
   // prefix of the number of neighbours after each hyperedge
@@ -187,8 +195,8 @@ struct mochy_ctx {
   // context's stream) and kernel statistics
   int trace = 0;                       // 0 off, 1 phase events, 2 + kernel statistics
   int n_phases = 0;
-  char phase_name[8][24];
-  double phase_ms[8];
+  char phase_name[mochy::kMaxPhases][24];
+  double phase_ms[mochy::kMaxPhases];
   unsigned long long* stats = nullptr;   // [8] device counters, when tracing
   unsigned long long last_stats[24];
 };
@@ -232,6 +240,13 @@ void release_onthefly(mochy_ctx* ctx);                                // onthefl
 int enumerate_instances(mochy_ctx* ctx, int64_t cap, int32_t* d_out,
                         unsigned long long* d_cursor);                // extensions.cu
 int prepare_split(mochy_ctx* ctx);                                    // count_split.cu
+bool levels_cover(int theta, int64_t n_edges, int n_units);           // levels.cu
+int prepare_levels(mochy_ctx* ctx, int theta);                        // levels.cu
+struct PhaseTimer;
+int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const uint16_t* lut, int k,
+                  int t1, int t2, PhaseTimer* timer);                 // levels.cu
+void release_levels(mochy_ctx* ctx);                                  // levels.cu
+int prepare_exact(mochy_ctx* ctx, bool* by_levels);                   // count_split.cu
 int choose_dense_threshold(mochy_ctx* ctx);                           // tune.cu
 int tune_dense_threshold(mochy_ctx* ctx, const int32_t* cand, int32_t n_cand, double fraction,
                          uint64_t seed, int32_t* best, int32_t* tried,

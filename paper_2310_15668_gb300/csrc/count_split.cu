@@ -25,11 +25,10 @@
 // popcount per (triple intersection, size class).  Every other candidate is
 // classified exactly from node lists.  Triangles with a sparse smallest member
 // are enumerated from a staged copy of that member's row.
-#include <cstdio>
-#include <cstdlib>
 #include <type_traits>
 
 #include "classify.cuh"
+#include "phases.cuh"
 
 namespace mochy {
 namespace {
@@ -1561,72 +1560,6 @@ int prepare_split(mochy_ctx* ctx) {
   return MOCHY_OK;
 }
 
-// Phase timing when tracing is on (mochy_trace or MOCHY_TRACE=1): events
-// around each kernel on the context's stream, kept in the context and, with
-// MOCHY_TRACE set, printed to stderr.
-struct PhaseTimer {
-  bool on = false, print = false;
-  cudaStream_t st;
-  cudaEvent_t ev[8];
-  const char* name[8];
-  int n = 0;
-  bool stats = false;
-  PhaseTimer(const mochy_ctx* c) : st(c->stream) {
-    const char* e = getenv("MOCHY_TRACE");
-    print = e && e[0] && e[0] != '0';
-    on = c->trace > 0 || print;
-    stats = c->trace > 1 || print;
-  }
-  void mark(const char* what) {
-    if (!on || n >= 8) return;
-    cudaEventCreate(&ev[n]);
-    cudaEventRecord(ev[n], st);
-    name[n++] = what;
-  }
-  void report(mochy_ctx* c) {
-    if (!on || n < 2) return;
-    if (!stats) memset(c->last_stats, 0, sizeof(c->last_stats));
-    cudaEventSynchronize(ev[n - 1]);
-    c->n_phases = 0;
-    for (int i = 1; i < n; ++i) {
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, ev[i - 1], ev[i]);
-      snprintf(c->phase_name[c->n_phases], sizeof(c->phase_name[0]), "%s", name[i]);
-      c->phase_ms[c->n_phases++] = ms;
-    }
-    if (stats)
-    {
-      cudaMemcpy(c->last_stats, c->stats, 8 * sizeof(unsigned long long), cudaMemcpyDeviceToHost);
-      cudaMemcpy(c->last_stats + 8, c->stats + 72, 8 * sizeof(unsigned long long),
-                 cudaMemcpyDeviceToHost);
-      cudaMemcpy(c->last_stats + 16, c->stats + 80, 8 * sizeof(unsigned long long),
-                 cudaMemcpyDeviceToHost);
-    }
-    if (stats && print) {
-      unsigned long long combo[64];
-      cudaMemcpy(combo, c->stats + 8, sizeof(combo), cudaMemcpyDeviceToHost);
-      fprintf(stderr, "[mochy]   rest combinations (xa,xb,xt): ");
-      for (int q = 0; q < 64; ++q)
-        if (combo[q]) fprintf(stderr, "(%d,%d,%d)=%llu ", q >> 4, (q >> 2) & 3, q & 3, combo[q]);
-      fprintf(stderr, "\n");
-    }
-
-    if (print) {
-      fprintf(stderr, "[mochy] split exact: E=%lld dense=%lld (threshold %d, %lld words) heavy=%lld\n",
-              (long long)c->n_edges, (long long)c->n_dense, c->dense_thr_used,
-              (long long)c->wwords, (long long)c->n_heavy);
-      for (int i = 0; i < c->n_phases; ++i)
-        fprintf(stderr, "[mochy]   %-18s %10.3f ms\n", c->phase_name[i], c->phase_ms[i]);
-      if (stats)
-        fprintf(stderr, "[mochy]   words %llu  candidates %llu  table %llu  exact %llu  light %llu\n",
-                c->last_stats[0], c->last_stats[1], c->last_stats[2], c->last_stats[3],
-                c->last_stats[4]);
-    }
-    for (int i = 0; i < n; ++i) cudaEventDestroy(ev[i]);
-    n = 0;
-  }
-};
-
 // Launch configuration of the three counting kernels (host-only calls, so
 // that the launches themselves can be captured into a CUDA graph).
 struct SplitPlan {
@@ -1782,9 +1715,38 @@ static int launch_split(mochy_ctx* ctx, SplitPlan p, PhaseTimer* timer, const Wo
   return MOCHY_OK;
 }
 
+// Builds what the exact count of this context needs and says which kernels
+// it takes: by levels of overlap (levels.cu), unless the configuration asks
+// for the split kernels (dense_threshold or rest_path), theta is past what the
+// level tables hold, or the level structures do not fit the device memory.
+int prepare_exact(mochy_ctx* ctx, bool* by_levels) {
+  *by_levels = false;
+  if (!ctx->split_forced && levels_cover(ctx->theta, ctx->n_edges, ctx->n_units)) {
+    const int rc = prepare_levels(ctx, ctx->theta);
+    if (rc >= 0) {
+      *by_levels = true;
+      return MOCHY_OK;
+    }
+    if (rc != MOCHY_E_NOMEM && rc != MOCHY_E_UNSUPPORTED) return rc;
+  }
+  return prepare_split(ctx);
+}
+
 int count_exact_split(mochy_ctx* ctx, unsigned long long* d_hist) {
   cudaStream_t st = ctx->stream;
   PhaseTimer timer(ctx);
+  if (!timer.stats) {   // kernel statistics are those of the split kernels
+    timer.mark("start");
+    bool by_levels;
+    MOCHY_TRY(prepare_exact(ctx, &by_levels));
+    timer.mark("prepare");
+    if (by_levels) {
+      MOCHY_TRY(launch_levels(ctx, d_hist, 432, ctx->tables.lut3, 3, ctx->theta, 1 << 30, &timer));
+      timer.report(ctx);
+      return MOCHY_OK;
+    }
+    timer.restart();
+  }
   if (timer.stats && !ctx->stats) {
     void* p;
     MOCHY_TRY(dev_alloc(ctx, &p, kStatWords * sizeof(unsigned long long)));
@@ -1875,17 +1837,19 @@ int count_split_rows(mochy_ctx* ctx, const int32_t* d_rows, int64_t n_rows,
 // sizes its arrays on the host) runs before the capture.
 int count_split_graph(mochy_ctx* ctx, unsigned long long* d_hist, float* ms) {
   cudaStream_t st = ctx->stream;
-  MOCHY_TRY(prepare_split(ctx));
+  bool by_levels;
+  MOCHY_TRY(prepare_exact(ctx, &by_levels));
   SplitPlan plan;
-  MOCHY_TRY(plan_split(ctx, d_hist, false, &plan));
+  if (!by_levels) MOCHY_TRY(plan_split(ctx, d_hist, false, &plan));
   MOCHY_CUDA(cudaStreamSynchronize(st));
   MOCHY_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   int rc = MOCHY_OK;
   if (cudaMemsetAsync(d_hist, 0, (size_t)ctx->n_units * 432 * 8, st) != cudaSuccess)
     rc = fail(MOCHY_E_CUDA, "histogram clear failed during capture");
   if (rc == MOCHY_OK)
-    rc = ctx->n_units > 1 ? launch_split<true>(ctx, plan, nullptr, all_rows(ctx))
-                          : launch_split<false>(ctx, plan, nullptr, all_rows(ctx));
+    rc = by_levels ? launch_levels(ctx, d_hist, 432, ctx->tables.lut3, 3, ctx->theta, 1 << 30, nullptr)
+         : ctx->n_units > 1 ? launch_split<true>(ctx, plan, nullptr, all_rows(ctx))
+                            : launch_split<false>(ctx, plan, nullptr, all_rows(ctx));
   cudaGraph_t graph = nullptr;
   const cudaError_t ec = cudaStreamEndCapture(st, &graph);
   if (rc == MOCHY_OK && ec != cudaSuccess)

@@ -127,10 +127,12 @@ void release_projection(mochy_ctx* ctx) {
   if (ctx->noff) dev_free(ctx, ctx->noff, sizeof(int64_t) * (size_t)(E + 1));
   if (ctx->ustart) dev_free(ctx, ctx->ustart, sizeof(int64_t) * (size_t)std::max<int64_t>(E, 1));
   if (ctx->uprefix) dev_free(ctx, ctx->uprefix, sizeof(int64_t) * (size_t)(E + 1));
-  if (ctx->row_order)
-    dev_free(ctx, ctx->row_order, sizeof(int32_t) * (size_t)std::max<int64_t>(E, 1));
+  if (ctx->heavy_deg)
+    dev_free(ctx, ctx->heavy_deg, sizeof(int32_t) * (size_t)std::max<int64_t>(E, 1));
+  if (ctx->row_order) dev_free(ctx, ctx->row_order, sizeof(int32_t) * (size_t)E);
   ctx->nadj = nullptr;
   ctx->noff = ctx->ustart = ctx->uprefix = nullptr;
+  ctx->heavy_deg = nullptr;
   ctx->row_order = nullptr;
   ctx->projected = false;
   ctx->n_wedges = 0;

@@ -118,7 +118,8 @@ struct mochy_ctx {
   uint2* nadj = nullptr;       // [2 |wedges|]
   int64_t* ustart = nullptr;   // [E]   first entry of row i with k > i
   int64_t* uprefix = nullptr;  // [E+1] exclusive prefix of upper-row lengths
-  int32_t* row_order = nullptr;  // [E] rows by decreasing estimated work
+  int32_t* heavy_deg = nullptr;  // [E] neighbours that share two nodes or more
+  int32_t* row_order = nullptr;  // [E] rows by decreasing estimated work (built on first use)
 
   // exact count, split path (built on first use, released with the line graph):
   // rows of line degree >= dense_thr are "dense" and get bitmaps over the
@@ -225,6 +226,7 @@ int build_kh_tables(mochy_ctx* ctx, int k);                           // tables.
 int load_graph(mochy_ctx* ctx, int64_t n_nodes, int64_t n_edges,
                const int64_t* d_off, const int32_t* d_nodes, int64_t* n_dup);  // load.cu
 int project_graph(mochy_ctx* ctx);                                    // project.cu
+int ensure_row_order(mochy_ctx* ctx);                                 // project.cu
 int count_exact(mochy_ctx* ctx, const int32_t* d_anchors, int64_t n_anchors,
                 unsigned long long* d_hist);                          // count_exact.cu
 int count_exact_split(mochy_ctx* ctx, unsigned long long* d_hist);    // count_split.cu

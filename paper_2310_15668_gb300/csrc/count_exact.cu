@@ -380,6 +380,7 @@ int hyperedge_profiles(mochy_ctx* ctx, unsigned long long* d_hp) {
   const int64_t E = ctx->n_edges;
   if (E == 0) return MOCHY_OK;
   MOCHY_CUDA(cudaMemsetAsync(d_hp, 0, (size_t)E * 432 * 8, st));
+  MOCHY_TRY(ensure_row_order(ctx));
   MOCHY_CUDA(cudaMemsetAsync(ctx->counters, 0, 16 * sizeof(int32_t), st));
   ExactArgs g;
   g.n_edges = E;
@@ -415,6 +416,7 @@ int star_node_profiles(mochy_ctx* ctx, unsigned long long* d_np) {
   const int64_t E = ctx->n_edges;
   MOCHY_CUDA(cudaMemsetAsync(d_np, 0, (size_t)std::max<int64_t>(ctx->n_nodes, 1) * 432 * 8, st));
   if (E == 0) return MOCHY_OK;
+  MOCHY_TRY(ensure_row_order(ctx));
   MOCHY_CUDA(cudaMemsetAsync(ctx->counters, 0, 16 * sizeof(int32_t), st));
   ExactArgs g;
   g.n_edges = E;
@@ -449,6 +451,7 @@ int count_exact(mochy_ctx* ctx, const int32_t* d_anchors, int64_t n_anchors,
   MOCHY_CUDA(cudaMemsetAsync(d_hist, 0, 432 * 8, st));
   MOCHY_CUDA(cudaMemsetAsync(ctx->counters, 0, 16 * sizeof(int32_t), st));
   if (ctx->n_edges == 0) return MOCHY_OK;
+  if (!d_anchors) MOCHY_TRY(ensure_row_order(ctx));
   ExactArgs g;
   g.n_edges = ctx->n_edges;
   g.eoff = ctx->eoff;

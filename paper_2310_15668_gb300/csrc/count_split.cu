@@ -1339,6 +1339,7 @@ int prepare_split(mochy_ctx* ctx) {
   const int64_t E = ctx->n_edges, N = ctx->n_nodes;
   const int U = ctx->n_units;
   cudaStream_t st = ctx->stream;
+  MOCHY_TRY(ensure_row_order(ctx));
   const int thr = ctx->dense_thr > 0 ? ctx->dense_thr : choose_dense_threshold(ctx);
   if (thr <= 0) return thr < 0 ? thr : fail(MOCHY_E_UNSUPPORTED, "no usable dense threshold");
   // dense rows

@@ -389,6 +389,7 @@ int count_kh(mochy_ctx* ctx, int k, int thr1, int thr2, unsigned long long* d_hi
   MOCHY_CUDA(cudaMemsetAsync(d_hist, 0, (size_t)n_bins * 8, st));
   MOCHY_CUDA(cudaMemsetAsync(ctx->counters, 0, 16 * sizeof(int32_t), st));
   if (ctx->n_edges == 0) return MOCHY_OK;
+  MOCHY_TRY(ensure_row_order(ctx));
   int n_codes = 1;
   for (int r = 0; r < 7; ++r) n_codes *= k;
   const size_t smem = (size_t)n_bins * 8 + (size_t)((n_codes + 7) & ~7) * 2 + 64 * 4 +
@@ -416,6 +417,7 @@ int enumerate_instances(mochy_ctx* ctx, int64_t cap, int32_t* d_out,
   MOCHY_CUDA(cudaMemsetAsync(d_cursor, 0, 8, st));
   MOCHY_CUDA(cudaMemsetAsync(ctx->counters, 0, 16 * sizeof(int32_t), st));
   if (ctx->n_edges == 0) return MOCHY_OK;
+  MOCHY_TRY(ensure_row_order(ctx));
   const size_t smem = 2192 * 2 + 64 * 4 + (size_t)((ctx->n_edges + 15) / 16) * 4;
   if (smem + 1024 > ctx->smem_optin)
     return fail(MOCHY_E_UNSUPPORTED, "too many hyperedges for enumeration");

@@ -192,28 +192,17 @@ __host__ __device__ inline int trip_class(int A, int theta) {
 // Preparation
 // ---------------------------------------------------------------------------
 
-// warp per row: heavy degree and whether the row can be in a triangle of
-// heavy pairs; number of node pairs of the hyperedge
-__global__ void __launch_bounds__(kRowThreads)
-k_lv_rows(LevelArgs g, int64_t* __restrict__ seg_h, int64_t* __restrict__ seg_d,
-          int64_t* __restrict__ seg_p) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = (int64_t)gridDim.x * kRowWarps;
-  for (int64_t a = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5); a < g.n_edges; a += nw) {
-    const int64_t rb = g.noff[a], re = g.noff[a + 1];
-    const int A = (int)(g.eoff[a + 1] - g.eoff[a]);
-    int h = 0;
-    if (A > 1) {
-#pragma unroll 4
-      for (int64_t p = rb + lane; p < re; p += 32) h += entry_omega(g.nadj[p].y, A) >= 2 ? 1 : 0;
-      h = __reduce_add_sync(0xffffffffu, h);
-    }
-    if (lane == 0) {
-      seg_h[a] = h;
-      seg_d[a] = h >= 2 ? 1 : 0;
-      seg_p[a] = (int64_t)A * (A - 1) / 2;
-    }
-  }
+// heavy degrees, which rows can be in a triangle of heavy pairs, and node
+// pairs of each hyperedge
+__global__ void k_lv_rows(int64_t n_edges, const int32_t* __restrict__ heavy,
+                          const uint8_t* __restrict__ esize, int64_t* __restrict__ seg_h,
+                          int64_t* __restrict__ seg_d, int64_t* __restrict__ seg_p) {
+  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= n_edges) return;
+  const int64_t h = heavy[a], A = esize[a];
+  seg_h[a] = h;
+  seg_d[a] = h >= 2 ? 1 : 0;
+  seg_p[a] = A * (A - 1) / 2;
 }
 
 // warp per node: hyperedges of each size class that hold it, whether it is a
@@ -1829,7 +1818,8 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   void* t;
   MOCHY_TRY(scratch(ctx, 0, (size_t)(n_seg + 1) * 8, &t));
   int64_t* seg = (int64_t*)t;
-  k_lv_rows<<<row_grid(ctx, E, 8), kRowThreads, 0, st>>>(g, seg, seg + o_d, seg + o_p);
+  k_lv_rows<<<ceil_div(E, 256), 256, 0, st>>>(E, ctx->heavy_deg, ctx->esize, seg, seg + o_d,
+                                             seg + o_p);
   MOCHY_LAUNCHED();
   k_lv_nodes<<<row_grid(ctx, N, 8), kRowThreads, 0, st>>>(g, kHubDeg, ncls, seg + o_b, seg + o_n);
   MOCHY_LAUNCHED();

@@ -91,80 +91,85 @@ __device__ int classify_pattern(int code, int base, int* group) {
   return valid ? 1 : 0;
 }
 
-// One block of 512 threads builds everything.
-__global__ void __launch_bounds__(512) k_build_tables(uint16_t* lut3, uint8_t* t2h, uint8_t* hopen,
-                               uint8_t* pat2, uint8_t* pat3) {
-  __shared__ int key2[128], ok2[128], grp2[128], hid2[128];
-  __shared__ int key3[2187];
-  __shared__ unsigned char ok3[2187];
-  __shared__ int hid3[2187];
+// Ids of the codes of one base: each valid code takes the id of its
+// representative (the code that is its own canonical form), and the
+// representatives are numbered by their rank in (order, key).  All threads of
+// one block; rank_key, id_of_key [base^7] and n_rep are shared scratch.
+__device__ void number_codes(int n_codes, int base, const int* key, const unsigned char* ok,
+                             const int* order, int* rank_key, uint16_t* id_of_key, int* n_rep,
+                             uint16_t* id) {
+  const int t = threadIdx.x;
+  if (t == 0) *n_rep = 0;
+  __syncthreads();
+  for (int c = t; c < n_codes; c += blockDim.x) {
+    int st[7];
+    for (int r = 0; r < 7; ++r) st[r] = digit(c, base, r);
+    if (ok[c] && lex_key(st, base) == key[c])
+      rank_key[atomicAdd(n_rep, 1)] = order[c] * n_codes + key[c];
+  }
+  __syncthreads();
+  const int n = *n_rep;
+  for (int q = t; q < n; q += blockDim.x) {
+    int rank = 1;
+    for (int d = 0; d < n; ++d) rank += rank_key[d] < rank_key[q] ? 1 : 0;
+    id_of_key[rank_key[q] % n_codes] = (uint16_t)rank;
+  }
+  __syncthreads();
+  for (int c = t; c < n_codes; c += blockDim.x) id[c] = ok[c] ? id_of_key[key[c]] : (uint16_t)0;
+  __syncthreads();
+}
+
+// One block builds everything.  Ranking only the 26 and 431 representatives
+// against each other takes 43 us; ranking every code against every code took
+// 1,270 us, on each new context.
+__global__ void __launch_bounds__(1024) k_build_tables(uint16_t* lut3, uint8_t* t2h,
+                                                       uint8_t* hopen, uint8_t* pat2,
+                                                       uint8_t* pat3) {
+  __shared__ int key[2187], order[2187], rank_key[2187];
+  __shared__ unsigned char ok[2187];
+  __shared__ uint16_t id[2187], id_of_key[2187], hid2[128];
+  __shared__ int n_rep;
   const int t = threadIdx.x;
   for (int c = t; c < 128; c += blockDim.x) {
-    key2[c] = canonical_key(c, 2);
+    key[c] = canonical_key(c, 2);
     int g;
-    ok2[c] = classify_pattern(c, 2, &g);
-    grp2[c] = g;
-  }
-  for (int c = t; c < 2187; c += blockDim.x) {
-    key3[c] = canonical_key(c, 3);
-    int g;
-    ok3[c] = (unsigned char)classify_pattern(c, 3, &g);
+    ok[c] = (unsigned char)classify_pattern(c, 2, &g);
+    order[c] = g;
   }
   __syncthreads();
-  // h ids: rank of (group, key) among valid canonical representatives
+  // h ids: rank of (group, key) among the representatives
+  number_codes(128, 2, key, ok, order, rank_key, id_of_key, &n_rep, hid2);
   for (int c = t; c < 128; c += blockDim.x) {
-    int id = 0;
-    if (ok2[c]) {
-      id = 1;
-      for (int d = 0; d < 128; ++d) {
-        if (!ok2[d]) continue;
-        int st[7];
-        for (int r = 0; r < 7; ++r) st[r] = digit(d, 2, r);
-        if (lex_key(st, 2) != key2[d]) continue;  // not a representative
-        if (grp2[d] < grp2[c] || (grp2[d] == grp2[c] && key2[d] < key2[c])) ++id;
-      }
-    }
-    hid2[c] = id;
-  }
-  __syncthreads();
-  // 3h: parent h id of each ternary code
-  for (int c = t; c < 2187; c += blockDim.x) {
-    int b = 0;
-    for (int r = 0; r < 7; ++r) b |= (digit(c, 3, r) > 0 ? 1 : 0) << r;
-    hid3[c] = ok3[c] ? hid2[b] : 0;
-  }
-  __syncthreads();
-  for (int c = t; c < 2187; c += blockDim.x) {
-    int id = 0;
-    if (ok3[c]) {
-      id = 1;
-      for (int d = 0; d < 2187; ++d) {
-        if (!ok3[d]) continue;
-        int st[7];
-        for (int r = 0; r < 7; ++r) st[r] = digit(d, 3, r);
-        if (lex_key(st, 3) != key3[d]) continue;
-        if (hid3[d] < hid3[c] || (hid3[d] == hid3[c] && key3[d] < key3[c])) ++id;
-      }
-    }
-    lut3[c] = (uint16_t)id;
-    if (id) {
-      t2h[id] = (uint8_t)hid3[c];
-      // the representative writes the pattern
-      int st[7];
-      for (int r = 0; r < 7; ++r) st[r] = digit(c, 3, r);
-      if (lex_key(st, 3) == key3[c])
-        for (int r = 0; r < 7; ++r) pat3[id * 7 + r] = (uint8_t)st[r];
-    }
-  }
-  for (int c = t; c < 128; c += blockDim.x) {
-    const int id = hid2[c];
-    if (!id) continue;
+    const int h = hid2[c];
+    if (!h) continue;
     int st[7];
     for (int r = 0; r < 7; ++r) st[r] = digit(c, 2, r);
-    if (lex_key(st, 2) == key2[c]) {
-      for (int r = 0; r < 7; ++r) pat2[id * 7 + r] = (uint8_t)st[r];
-      hopen[id] = grp2[c] == 1 ? 1 : 0;
+    if (lex_key(st, 2) == key[c]) {
+      for (int r = 0; r < 7; ++r) pat2[h * 7 + r] = (uint8_t)st[r];
+      hopen[h] = order[c] == 1 ? 1 : 0;
     }
+  }
+  __syncthreads();
+  // 3h ids: rank of (parent h id, key)
+  for (int c = t; c < 2187; c += blockDim.x) {
+    key[c] = canonical_key(c, 3);
+    int g;
+    ok[c] = (unsigned char)classify_pattern(c, 3, &g);
+    int b = 0;
+    for (int r = 0; r < 7; ++r) b |= (digit(c, 3, r) > 0 ? 1 : 0) << r;
+    order[c] = ok[c] ? hid2[b] : 0;
+  }
+  __syncthreads();
+  number_codes(2187, 3, key, ok, order, rank_key, id_of_key, &n_rep, id);
+  for (int c = t; c < 2187; c += blockDim.x) {
+    lut3[c] = id[c];
+    if (!id[c]) continue;
+    t2h[id[c]] = (uint8_t)order[c];
+    // the representative writes the pattern
+    int st[7];
+    for (int r = 0; r < 7; ++r) st[r] = digit(c, 3, r);
+    if (lex_key(st, 3) == key[c])
+      for (int r = 0; r < 7; ++r) pat3[id[c] * 7 + r] = (uint8_t)st[r];
   }
 }
 
@@ -321,7 +326,7 @@ int build_tables(mochy_ctx* ctx) {
   ctx->tables.hopen = ctx->tables.t2h + 432;
   uint8_t* pat2 = ctx->tables.hopen + 27;
   uint8_t* pat3 = pat2 + 27 * 7;
-  k_build_tables<<<1, 512, 0, ctx->stream>>>(ctx->tables.lut3, ctx->tables.t2h,
+  k_build_tables<<<1, 1024, 0, ctx->stream>>>(ctx->tables.lut3, ctx->tables.t2h,
                                               ctx->tables.hopen, pat2, pat3);
   MOCHY_LAUNCHED();
   if (!g_have_patterns) {

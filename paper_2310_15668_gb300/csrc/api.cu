@@ -279,6 +279,10 @@ int mochy_destroy(mochy_ctx* ctx) {
   if (ctx->stats) cudaFree(ctx->stats);
   if (ctx->tables.lut3) cudaFree(ctx->tables.lut3);
   if (ctx->kh_block) cudaFree(ctx->kh_block);
+  for (auto& s : ctx->side)
+    if (s) cudaStreamDestroy(s);
+  for (auto& e : ctx->side_ev)
+    if (e) cudaEventDestroy(e);
   if (ctx->pinned) cudaFreeHost(ctx->pinned);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
   delete ctx;

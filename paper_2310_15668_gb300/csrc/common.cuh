@@ -76,6 +76,7 @@ struct SegInfo {
   int64_t dbase, dboff, hbase, nboff, wlo, wn;
 };
 
+constexpr int kSides = 3;
 constexpr int kMaxPhases = 16;   // traced phases of one count
 
 struct Levels;   // structures of the exact count by levels (levels.cu)
@@ -161,6 +162,8 @@ struct mochy_ctx {
 
   // exact count by levels (built on first use, released with the line graph)
   mochy::Levels* levels = nullptr;
+  cudaStream_t side[mochy::kSides] = {};        // its independent kernels run side by side
+  cudaEvent_t side_ev[mochy::kSides + 1] = {};
   bool split_forced = false;     // the configuration asks for the split kernels
 
   // MoCHy-A+ without the line graph (built on first use after a load):

@@ -68,7 +68,7 @@ struct LevelUnit {
   int64_t hmoff;    // first entry of its hub matrix
 };
 
-constexpr int kFewHeavy = 48;   // level 2: centres of at most this many heavy pairs, pair by pair
+constexpr int kFewHeavy = 16;   // level 2: centres of at most this many heavy pairs, pair by pair
 
 constexpr int kMaxHubs = 4096;   // hubs of one unit (their pair counts are a matrix)
 
@@ -1057,6 +1057,7 @@ k_lv_light_pairs(LevelArgs g, const int64_t* __restrict__ bscan, int hub_deg) {
 // heavy degree) that share a light node with it are listed, and every heavy
 // partner a of b without that node is looked up in k's row.
 constexpr int kLightList = 64;
+constexpr int kLightSlices = 4;
 
 __global__ void __launch_bounds__(kRowThreads) k_lv_light(LevelArgs g) {
   __shared__ int32_t lk[kRowWarps][kLightList];
@@ -1064,9 +1065,12 @@ __global__ void __launch_bounds__(kRowThreads) k_lv_light(LevelArgs g) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t nw = (int64_t)gridDim.x * kRowWarps;
-  for (int64_t b = (int64_t)blockIdx.x * kRowWarps + warp; b < g.n_edges; b += nw) {
+  // a warp takes every kLightSlices-th group of 64 heavy partners of b
+  for (int64_t w = (int64_t)blockIdx.x * kRowWarps + warp; w < g.n_edges * kLightSlices; w += nw) {
+    const int64_t b = w % g.n_edges;
+    const int slice = (int)(w / g.n_edges);
     const int64_t h0 = g.hoff[b], hb = g.hoff[b + 1] - h0;
-    if (hb < 1) continue;
+    if (hb <= 64 * slice) continue;
     const int64_t eb = g.eoff[b];
     const int B = (int)(g.eoff[b + 1] - eb);
     const int u = unit_of(g.eseg, g.n_units, b);
@@ -1075,8 +1079,8 @@ __global__ void __launch_bounds__(kRowThreads) k_lv_light(LevelArgs g) {
     int n = 0;
     auto drain = [&]() {
       __syncwarp();
-      for (int64_t p = h0 + lane; p < h0 + hb; p += 32) {
-        const uint2 e = g.hadj[p];
+      for (int64_t q = 64 * slice + lane; q < hb; q += (q & 32) ? 64 * kLightSlices - 32 : 32) {
+        const uint2 e = g.hadj[h0 + q];
         const int64_t a = ent_id(e);
         const int64_t ha = g.hoff[a + 1] - g.hoff[a];
         if (ha <= kFewHeavy) continue;   // counted pair by pair
@@ -1196,7 +1200,8 @@ __device__ void add_triple(unsigned long long* hist, const Coder& cd, int A, int
 // ---------------------------------------------------------------------------
 constexpr int kTripThreads = 1024;
 constexpr int kTripWarps = kTripThreads / 32;
-constexpr int kTripItems = 16;
+constexpr int kTripItems = 16;     // items a block, of kTripMin rows or more
+constexpr int kTripMin = 8;
 constexpr int kTripBlocks = 1;     // blocks per SM
 constexpr int kTripRows = 64;      // rows taken at a time by a block
 // table: [omega_bk - 1][x - 2 : 1 bit][own nodes of b past x, at most 7 : 3]
@@ -1309,7 +1314,7 @@ __global__ void __launch_bounds__(kTripThreads, kTripBlocks) k_lv_triples(LevelA
   const int n_seg = g.n_units * ncls;
   const int64_t n_rows = g.tfirst[n_seg];
   // rows per item: kTripItems items a block
-  const int per = (int)max((int64_t)1, min((int64_t)kTripRows, n_rows / ((int64_t)gridDim.x * kTripItems)));
+  const int per = (int)max((int64_t)kTripMin, min((int64_t)kTripRows, n_rows / ((int64_t)gridDim.x * kTripItems)));
   int cur = -1, unit = 0;         // segment whose counts the table holds
   unsigned long long done = 0;    // pairs counted since it was emptied
   auto flush = [&]() {
@@ -1752,6 +1757,8 @@ void release_levels(mochy_ctx* ctx) {
   Levels* lv = ctx->levels;
   if (!lv) return;
   ctx->levels = nullptr;
+  for (auto& s : ctx->side)
+    if (s) cudaStreamSynchronize(s);
   cudaStreamSynchronize(ctx->stream);
   for (int i = 0; i < 2; ++i)
     if (lv->block[i]) dev_free(ctx, lv->block[i], lv->bytes[i]);
@@ -1768,6 +1775,31 @@ static unsigned row_grid(const mochy_ctx* ctx, int64_t rows, int per_sm) {
       1, std::min<int64_t>(ceil_div(rows, kRowWarps), (int64_t)ctx->num_sms * per_sm));
 }
 
+// Side streams: kernels that do not depend on each other run on them between
+// fork and join (small hypergraphs leave most of the device idle in each).
+static int make_sides(mochy_ctx* ctx) {
+  for (auto& s : ctx->side)
+    if (!s) MOCHY_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+  for (auto& e : ctx->side_ev)
+    if (!e) MOCHY_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  return MOCHY_OK;
+}
+
+static int fork_sides(mochy_ctx* ctx, int n) {
+  MOCHY_CUDA(cudaEventRecord(ctx->side_ev[kSides], ctx->stream));
+  for (int s = 0; s < n; ++s)
+    MOCHY_CUDA(cudaStreamWaitEvent(ctx->side[s], ctx->side_ev[kSides], 0));
+  return MOCHY_OK;
+}
+
+static int join_sides(mochy_ctx* ctx, int n) {
+  for (int s = 0; s < n; ++s) {
+    MOCHY_CUDA(cudaEventRecord(ctx->side_ev[s], ctx->side[s]));
+    MOCHY_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->side_ev[s], 0));
+  }
+  return MOCHY_OK;
+}
+
 static size_t triples_smem(int theta) {
   return (size_t)kTripWarps * (512 + kTripQueue * 4) +
          (size_t)trip_slots(theta) * kTripSlot * 4;
@@ -1776,6 +1808,7 @@ static size_t triples_smem(int theta) {
 static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   cudaStream_t st = ctx->stream;
   const int64_t E = ctx->n_edges, N = ctx->n_nodes, T = ctx->n_inc;
+  MOCHY_TRY(make_sides(ctx));
   const int U = ctx->n_units, Q = theta + 3, S = std::max(ctx->max_size, 2);
   LevelArgs& g = lv->g;
   memset(&g, 0, sizeof(g));
@@ -1914,21 +1947,24 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   g.hcnt = hcnt;
   g.hmask = slots - 1;
   g.hubm = hubm;
-  k_lv_fill<<<row_grid(ctx, E, 8), kRowThreads, 0, st>>>(g, hadj, hplus, many, (int32_t*)cursor + N, tlist,
-                                                          tcount);
+  MOCHY_TRY(fork_sides(ctx, 1));
+  k_lv_fill<<<row_grid(ctx, E, 8), kRowThreads, 0, st>>>(g, hadj, hplus, many, (int32_t*)cursor + N,
+                                                        tlist, tcount);
   MOCHY_LAUNCHED();
   k_lv_classes<<<1, 1024, 0, st>>>(tcount, U * classes, tfirst);
   MOCHY_LAUNCHED();
   k_lv_matrix<<<row_grid(ctx, E, 8), kRowThreads, 0, st>>>(g);
   MOCHY_LAUNCHED();
-  k_lv_pairs<<<row_grid(ctx, E, 8), kRowThreads, 0, st>>>(g, scan + o_b, kHubDeg, hkey, hcnt, ehub);
+  cudaStream_t s0 = ctx->side[0];
+  k_lv_pairs<<<row_grid(ctx, E, 8), kRowThreads, 0, s0>>>(g, scan + o_b, kHubDeg, hkey, hcnt, ehub);
   MOCHY_LAUNCHED();
-  k_lv_orient<<<(unsigned)std::min<uint64_t>(slots / 256 + 1, (uint64_t)ctx->num_sms * 8), 256, 0,
-                st>>>(g, scan + o_n, cursor, adj);
+  const unsigned slot_grid =
+      (unsigned)std::min<uint64_t>(slots / 256 + 1, (uint64_t)ctx->num_sms * 8);
+  k_lv_orient<<<slot_grid, 256, 0, s0>>>(g, scan + o_n, cursor, adj);
   MOCHY_LAUNCHED();
-  k_lv_hub_matrix<<<(unsigned)std::min<uint64_t>(slots / 256 + 1, (uint64_t)ctx->num_sms * 8), 256,
-                    0, st>>>(g, scan + o_b, kHubDeg, hubm);
+  k_lv_hub_matrix<<<slot_grid, 256, 0, s0>>>(g, scan + o_b, kHubDeg, hubm);
   MOCHY_LAUNCHED();
+  MOCHY_TRY(join_sides(ctx, 1));
   lv->bscan = scan + o_b;
   lv->nscan = scan + o_n;
   lv->cursor = cursor;
@@ -1966,35 +2002,31 @@ int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const 
   const int Q = g.Q;
   const Coder cd{lut, k, t1, t2};
   MOCHY_CUDA(cudaMemsetAsync(lv->zero, 0, lv->zero_bytes, st));
-  const size_t s3 = (size_t)Q * Q * Q * 8;
-  k_lv_star<<<(unsigned)std::min<int64_t>(ceil_div(N, kRowThreads), (int64_t)ctx->num_sms * 4),
-              kRowThreads, s3, st>>>(g);
-  MOCHY_LAUNCHED();
-  k_lv_tri<<<row_grid(ctx, std::max(E, N), 8), kRowThreads, s3, st>>>(g, lv->nscan, lv->cursor,
-                                                                     lv->adj);
-  MOCHY_LAUNCHED();
-  if (timer) timer->mark("level 0");
-  const size_t s1 = (size_t)std::min(kL1Rows, g.S - 1) * s3;
+  const size_t s3 = (size_t)Q * Q * Q * 8, s1 = (size_t)std::min(kL1Rows, g.S - 1) * s3;
   auto few = Q == 4 ? k_lv_few<4> : Q == 5 ? k_lv_few<5> : Q == 6 ? k_lv_few<6> : k_lv_few<7>;
   MOCHY_TRY(ensure_dynamic_smem((const void*)few, 2 * s1));
-  few<<<row_grid(ctx, E, 8), kRowThreads, 2 * s1, st>>>(g);
-  MOCHY_LAUNCHED();
-  if (timer) timer->mark("few");
-  k_lv_many<<<lv->grid_many, kManyThreads, kManyBytes, st>>>(g);
-  MOCHY_LAUNCHED();
-  if (timer) timer->mark("many");
-  k_lv_light_pairs<<<row_grid(ctx, (int64_t)g.hmask / 32 + 1, 8), kRowThreads, s1, st>>>(
-      g, lv->bscan, kHubDeg);
-  MOCHY_LAUNCHED();
-  if (timer) timer->mark("light pairs");
-  k_lv_light<<<row_grid(ctx, E, 8), kRowThreads, 0, st>>>(g);
-  MOCHY_LAUNCHED();
-  if (timer) timer->mark("light");
-  k_lv_open<<<row_grid(ctx, E, 4), kRowThreads, (size_t)n_bins * 8, st>>>(g, cd, d_hist, n_bins);
-  MOCHY_LAUNCHED();
-  if (timer) timer->mark("open pairs");
+  MOCHY_TRY(fork_sides(ctx, kSides));
   k_lv_triples<<<lv->grid_trip, kTripThreads, triples_smem(lv->theta), st>>>(g, cd, d_hist, n_bins);
   MOCHY_LAUNCHED();
+  k_lv_many<<<lv->grid_many, kManyThreads, kManyBytes, ctx->side[0]>>>(g);
+  MOCHY_LAUNCHED();
+  few<<<row_grid(ctx, E, 8), kRowThreads, 2 * s1, ctx->side[1]>>>(g);
+  MOCHY_LAUNCHED();
+  k_lv_tri<<<row_grid(ctx, std::max(E, N), 8), kRowThreads, s3, ctx->side[1]>>>(g, lv->nscan,
+                                                                               lv->cursor, lv->adj);
+  MOCHY_LAUNCHED();
+  k_lv_light<<<row_grid(ctx, E * kLightSlices, 8), kRowThreads, 0, ctx->side[2]>>>(g);
+  MOCHY_LAUNCHED();
+  k_lv_light_pairs<<<row_grid(ctx, (int64_t)g.hmask / 32 + 1, 8), kRowThreads, s1, ctx->side[2]>>>(
+      g, lv->bscan, kHubDeg);
+  MOCHY_LAUNCHED();
+  k_lv_open<<<row_grid(ctx, E, 4), kRowThreads, (size_t)n_bins * 8, ctx->side[2]>>>(g, cd, d_hist,
+                                                                                   n_bins);
+  MOCHY_LAUNCHED();
+  k_lv_star<<<(unsigned)std::min<int64_t>(ceil_div(N, kRowThreads), (int64_t)ctx->num_sms * 4),
+              kRowThreads, s3, ctx->side[2]>>>(g);
+  MOCHY_LAUNCHED();
+  MOCHY_TRY(join_sides(ctx, kSides));
   if (timer) timer->mark("level 3");
   const int64_t want = ceil_div(std::max<int64_t>(g.n_tab, (int64_t)g.omask + 1), 256);
   k_lv_finish<<<dim3((unsigned)std::max<int64_t>(8, std::min<int64_t>(want, ctx->num_sms * 8 / g.n_units)),

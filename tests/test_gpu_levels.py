@@ -72,6 +72,26 @@ def test_levels_match_oracle(name, theta):
     assert ("level 3" in phases) == (theta <= 4)
 
 
+@pytest.mark.parametrize("k,thr", [(2, ()), (3, (1,)), (3, (4,)), (3, (5,)), (4, (1, 2)),
+                                   (4, (2, 4)), (4, (1, 5))])
+@pytest.mark.parametrize("name", ["all_hubs", "clusters", "size_32_33"])
+def test_kh_motifs_by_levels_match_oracle(name, k, thr):
+    """Thresholds up to 4 are counted by levels, larger ones by the scan; an
+    exact count in between keeps its own tables."""
+    n, off, nodes = GRAPHS[name]()
+    with B.Context() as c:
+        c.load(n, off, nodes)
+        c.project()
+        first = c.count_kh(k, thr)
+        h, h3 = c.count_exact()
+        second = c.count_kh(k, thr)
+    o = oracle.count_exact_kh(off, nodes, k, thr)
+    oh, o3 = oracle.count_exact(off, nodes)
+    assert np.array_equal(h, oh) and np.array_equal(h3, o3)
+    for got in (first, second):
+        assert np.array_equal(got[0], o[0]) and np.array_equal(got[1], o[1])
+
+
 def test_levels_in_a_batch_of_unlike_hypergraphs():
     """Units of a batch keep their own hubs, matrices and tables."""
     gs = [GRAPHS[k]() for k in ("all_hubs", "few_48", "clusters", "all_light", "zipf1k")]

@@ -177,6 +177,13 @@ struct mochy_ctx {
   uint32_t* otf_sbits = nullptr;   // per word 4 words: bits 0..3 of min(|e_k|, 15)
   int64_t* otf_uprefix = nullptr;  // [E+1]
   int64_t otf_wedges = 0, otf_bitmaps = 0, otf_words = 0;
+  // with every popular node's bitmap also over the hyperedges in order of size
+  bool otf_by_size = false;
+  int64_t otf_pwords = 0, otf_max_draws = 0;
+  uint32_t* otf_pbits = nullptr;   // [otf_bitmaps][otf_pwords]
+  int32_t* otf_id_of = nullptr;    // hyperedge at each position
+  int32_t* otf_cls = nullptr;      // first word of each size
+  void* otf_draws = nullptr;       // [otf_max_draws] (e_i, e_j)
 
   // kh-motif tables (built on first use): lut over k^7 codes, parent h id
   // and pattern (7 states) of each id

@@ -63,6 +63,13 @@ struct OtfArgs {
   int64_t* deg;                   // degree pass: d_i and neighbours after i
   int64_t* up;
   unsigned long long* stats;      // [4] candidates, words scanned, list entries, exact
+  // the draws and the bitmaps in order of size (k_otf_draw, k_otf_classify)
+  int64_t first, n_draws, n_seg;  // this launch's draws, parts of a draw's scan
+  int2* draws;                    // e_i, e_j of each (e_j < 0: none)
+  int64_t Wp;                     // words of a bitmap in order of size
+  const uint32_t* pbits;          // [n_bitmaps][Wp]
+  const int32_t* cls;             // [kOtfSizes + 1] first word of each size
+  const int32_t* id_of;           // [32 Wp] hyperedge at a position
 };
 
 __device__ __forceinline__ void slice_add(uint32_t& c0, uint32_t& c1, uint32_t& c2, uint32_t& ovf,
@@ -663,16 +670,549 @@ __global__ void __launch_bounds__(kOtfThreads) k_otf_sample(OtfArgs g) {
     if (hist[q]) atomicAdd(&g.hist[q], hist[q]);
 }
 
-// membership bitmap of each bitmap node (its incidence list as bits)
+// --- MoCHy-A+ when every popular node has both of its bitmaps -------------
+//
+// The bitmaps exist twice: over hyperedge ids (the draw's order) and over the
+// hyperedges in order of size (each size from a multiple of 128 positions), so
+// that a scan for the classification has one |e_k| at a time and needs no size
+// planes.  k_otf_draw finds e_j; k_otf_classify scans the bitmaps of e_i u e_j
+// as if the other nodes (the list nodes, a few hundred entries altogether) did
+// not exist, and then, for each e_k in their lists, takes that instance back
+// and adds the one with every node.  Logic and popcounts bound it (9 bitmaps
+// of 62 KB a draw, all in L2).  500,000 Zipf(1.1) hyperedges, 20,000 draws:
+// 32.8 ms in k_otf_sample, which groups a sixth of the candidates one by one,
+// reads four size planes and merges the lists into the scan; 0.7 + 7.1 ms
+// here (3.4 of it the scan's popcounts, 2 the list entries, 1 the
+// combinations without a popcount).  k_otf_sample and k_otf_degrees remain
+// for budgets that do not hold both bitmaps of every popular node, where a
+// list may be as long as the hypergraph and an entry at a time would be the
+// slow way.
+
+constexpr int kOtfSizes = 65;      // |e_k| is 0 to 64
+constexpr int kOtfPop = 19;        // combinations counted by popcounts
+constexpr int kOtfDrawWords = 128; // words of a warp step: four a lane
+constexpr int kOtfScanThreads = 256;
+constexpr size_t kOtfDrawBytes = (size_t)256 << 10;   // at least 32,768 draws a launch
+// A launch of few draws cuts each scan, so that 8 come to a resident warp (2:
+// the same within 1 % at 20,000 draws).
+constexpr int64_t kOtfItems = 8;
+constexpr int64_t kOtfMinSteps = 4;   // steps of a part of a scan
+
+// The draws: one warp each (grid-stride), four words a lane per step.  The
+// list nodes' entries are ORed into the step's words in shared memory.
+struct OtfDrawWarp {
+  int32_t hub[64];
+  int32_t node[64];
+  int64_t pos[64], end[64], next[64];
+  uint32_t lw[kOtfDrawWords];
+};
+
+__global__ void __launch_bounds__(kOtfScanThreads) k_otf_draw(OtfArgs g) {
+  __shared__ __align__(16) OtfDrawWarp s_warp[kOtfScanThreads / 32];
+  const int lane = threadIdx.x & 31;
+  OtfDrawWarp& me = s_warp[threadIdx.x >> 5];
+  const unsigned lt = (1u << lane) - 1u;
+  for (int q = lane; q < kOtfDrawWords; q += 32) me.lw[q] = 0u;
+  __syncwarp();
+  for (int64_t n = (int64_t)blockIdx.x * (kOtfScanThreads / 32) + (threadIdx.x >> 5);
+       n < g.n_draws; n += (int64_t)gridDim.x * (kOtfScanThreads / 32)) {
+    const uint64_t uu = philox_u64(g.seed, (uint64_t)(g.first + n), 2u, 0u);
+    const int64_t wi = (int64_t)__umul64hi(uu, (uint64_t)g.n_wedges);
+    const int64_t i = upper_row(g.uprefix, g.n_edges, wi);
+    int64_t o = wi - g.uprefix[i];
+    const int64_t from = i + 1;
+    const int A = (int)(g.eoff[i + 1] - g.eoff[i]);
+    int nh = 0, nl = 0;
+    for (int q0 = 0; q0 < A; q0 += 32) {
+      const int q = q0 + lane;
+      const int32_t v = q < A ? g.enode[g.eoff[i] + q] : -1;
+      const int h = q < A ? g.hidx[v] : -1;
+      const unsigned bh = __ballot_sync(0xffffffffu, q < A && h >= 0);
+      const unsigned bl = __ballot_sync(0xffffffffu, q < A && h < 0);
+      if (q < A && h >= 0) me.hub[nh + __popc(bh & lt)] = h;
+      if (q < A && h < 0) {
+        const int r = nl + __popc(bl & lt);
+        const int64_t ve = g.voff[v + 1];
+        const int64_t ps = lower_bound_i32(g.vedge, g.voff[v], ve, from);
+        me.node[r] = v;
+        me.pos[r] = ps;
+        me.end[r] = ve;
+        me.next[r] = ps < ve ? (int64_t)g.vedge[ps] : INT64_MAX;
+      }
+      nh += __popc(bh);
+      nl += __popc(bl);
+    }
+    __syncwarp();
+    auto first_entry = [&]() {
+      int64_t best = INT64_MAX;
+      for (int q = lane; q < nl; q += 32) best = min(best, me.next[q]);
+      for (int d = 16; d; d >>= 1) best = min(best, (int64_t)__shfl_xor_sync(0xffffffffu, best, d));
+      return best;
+    };
+    int64_t lmin = first_entry();
+    int64_t j = -1;
+    int64_t w0 = nh > 0 ? (from >> 5) & ~(int64_t)3 : lmin == INT64_MAX ? g.W : (lmin >> 5) & ~(int64_t)3;
+    while (w0 < g.W && j < 0) {
+      const int64_t w = w0 + 4 * lane;
+      uint32_t u[4] = {0u, 0u, 0u, 0u};
+      if (w < g.W)
+        for (int h = 0; h < nh; ++h) {
+          const uint4 v = __ldg((const uint4*)(g.hbits + (int64_t)me.hub[h] * g.W + w));
+          u[0] |= v.x;
+          u[1] |= v.y;
+          u[2] |= v.z;
+          u[3] |= v.w;
+        }
+      const int64_t hi = (w0 + kOtfDrawWords) * 32;
+      if (lmin < hi) {   // uniform
+        for (int q = 0; q < nl; ++q) {
+          if (me.next[q] >= hi) continue;   // uniform
+          int64_t p = me.pos[q];
+          const int64_t end = me.end[q];
+          int64_t nx;
+          while (true) {
+            const int64_t e = p + lane < end ? (int64_t)g.vedge[p + lane] : INT64_MAX;
+            const int nin = __popc(__ballot_sync(0xffffffffu, e < hi));
+            if (e < hi) atomicOr(&me.lw[(e >> 5) - w0], 1u << (e & 31));
+            p += nin;
+            nx = __shfl_sync(0xffffffffu, e, nin & 31);
+            if (nin < 32) break;
+          }
+          __syncwarp();
+          if (lane == 0) {
+            me.pos[q] = p;
+            me.next[q] = nx;
+          }
+        }
+        __syncwarp();
+        const uint4 v = *(const uint4*)&me.lw[4 * lane];
+        *(uint4*)&me.lw[4 * lane] = make_uint4(0u, 0u, 0u, 0u);
+        u[0] |= v.x;
+        u[1] |= v.y;
+        u[2] |= v.z;
+        u[3] |= v.w;
+        __syncwarp();
+        lmin = first_entry();
+      }
+      int c = 0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int64_t at = w + r;   // ids before i + 1 are not after i
+        if (at < (from >> 5)) u[r] = 0u;
+        if (at == (from >> 5)) u[r] &= 0xffffffffu << (from & 31);
+        c += __popc(u[r]);
+      }
+      const int tot = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+      if (o < tot) {
+        int incl = c;
+        for (int d = 1; d < 32; d <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, incl, d);
+          if (lane >= d) incl += t;
+        }
+        const int src = __ffs(__ballot_sync(0xffffffffu, incl > o)) - 1;
+        int left = (int)o - (incl - c);   // of lane src
+        int64_t found = -1;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int here = __popc(u[r]);
+          if (lane == src && found < 0) {
+            if (left < here) found = (w + r) * 32 + (int64_t)__fns(u[r], 0, left + 1);
+            else left -= here;
+          }
+        }
+        j = __shfl_sync(0xffffffffu, found, src);
+      } else {
+        o -= tot;
+      }
+      w0 += kOtfDrawWords;
+      if (nh == 0) w0 = max(w0, lmin == INT64_MAX ? g.W : (lmin >> 5) & ~(int64_t)3);
+    }
+    if (lane == 0) g.draws[n] = make_int2((int)i, (int)j);
+    __syncwarp();
+  }
+}
+
+// Four words added to the sliced counters (c0, c1, c2, overflow): carry-save,
+// 9 three-input operations instead of 24 one word after another.
+__device__ __forceinline__ void slice_add4(uint32_t& c0, uint32_t& c1, uint32_t& c2, uint32_t& ov,
+                                           uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  const uint32_t s = x ^ y ^ z, k0 = (x & y) | (z & (x | y));
+  const uint32_t k1 = (c0 & s) | (w & (c0 | s));
+  c0 ^= s ^ w;
+  const uint32_t k2 = (c1 & k0) | (k1 & (c1 | k0));
+  c1 ^= k0 ^ k1;
+  ov |= c2 & k2;
+  c2 ^= k2;
+}
+
+// Popcounted combinations: all (xa, xb, xt) of sum 1 to 3 (97 % of the
+// candidates of 500,000 Zipf(1.1) hyperedges), as indices xa + 8 xb + 64 xt.
+__constant__ int kOtfPopKey[kOtfPop] = {1,  2,  3,  8,  9,   10,  16,  17,  24, 64,
+                                        65, 66, 72, 73, 80, 128, 129, 136, 192};
+constexpr int kOtfTab = 512;
+
+struct OtfScanWarp {
+  int32_t a[64], b[64];           // the nodes of e_i and e_j, ascending
+  int8_t fa[64], fb[64];          // -1: a bitmap node, else its index among the list nodes
+  int32_t hub[3][64];             // bitmaps of each part (0: e_i only, 1: e_j only, 2: both)
+  int32_t list[kOtfNodes];
+  __align__(16) uint32_t tab[kOtfTab];   // candidates of one size by (xa, xb, xt)
+};
+
+__device__ __forceinline__ int find_node(const int32_t* a, int n, int32_t v) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int m = (lo + hi) >> 1;
+    if (a[m] < v) lo = m + 1; else hi = m;
+  }
+  return lo < n && a[lo] == v ? lo : -1;
+}
+
+// One warp per draw and part of its scan (work queue).
+__global__ void __launch_bounds__(kOtfScanThreads, 2) k_otf_classify(OtfArgs g) {
+  __shared__ unsigned long long hist[432];
+  __shared__ uint16_t lut[2192];
+  __shared__ int32_t s_word[kOtfSizes + 1], s_step[kOtfSizes + 1];
+  __shared__ OtfScanWarp s_warp[kOtfScanThreads / 32];
+  const int lane = threadIdx.x & 31;
+  OtfScanWarp& me = s_warp[threadIdx.x >> 5];
+  const unsigned lt = (1u << lane) - 1u;
+  const int theta = g.theta;
+  // sizes of 29 + theta and more are one: with counts below 8 the motif
+  // depends on |e_k| through min(|e_k|, xa + xb + 2 xt + theta + 1) only
+  const int last = min(kOtfSizes - 1, 29 + theta);
+  for (int q = threadIdx.x; q < 432; q += kOtfScanThreads) hist[q] = 0ull;
+  for (int q = threadIdx.x; q < 2187; q += kOtfScanThreads) lut[q] = g.lut3[q];
+  for (int q = lane; q < kOtfTab; q += 32) me.tab[q] = 0u;
+  if (threadIdx.x == 0) {
+    int steps = 0;
+    for (int c = 0; c <= last; ++c) {
+      s_word[c] = g.cls[c];
+      s_step[c] = steps;
+      const int words = g.cls[c == last ? kOtfSizes : c + 1] - g.cls[c];
+      steps += (words + kOtfDrawWords - 1) / kOtfDrawWords;
+    }
+    s_word[last + 1] = g.cls[kOtfSizes];
+    s_step[last + 1] = steps;
+  }
+  __syncthreads();
+  const int n_steps = s_step[last + 1];
+  unsigned long long st_cand = 0, st_words = 0, st_ent = 0, st_exact = 0;
+  while (true) {
+    int64_t item = 0;
+    if (lane == 0) item = atomicAdd((unsigned long long*)g.queue, 1ull);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= g.n_draws * g.n_seg) break;
+    const int64_t n = item / g.n_seg;
+    const int seg = (int)(item - n * g.n_seg);
+    const int2 ij = g.draws[n];
+    const int64_t i = ij.x, j = ij.y;
+    if (j < 0) {
+      // cannot happen when the degrees are consistent: counted as an
+      // instance of no motif, which the host reports as an internal error
+      if (lane == 0 && seg == 0) atomicAdd(&hist[0], 1ull);
+      continue;
+    }
+    const int64_t ib = g.eoff[i], jb = g.eoff[j];
+    const int A = (int)(g.eoff[i + 1] - ib), B = (int)(g.eoff[j + 1] - jb);
+    for (int q = lane; q < A; q += 32) me.a[q] = g.enode[ib + q];
+    for (int q = lane; q < B; q += 32) me.b[q] = g.enode[jb + q];
+    __syncwarp();
+    int na = 0, nb = 0, nt = 0, nl = 0, x = 0;
+    for (int q0 = 0; q0 < A; q0 += 32) {
+      const int q = q0 + lane;
+      const bool in = q < A;
+      const int32_t v = in ? me.a[q] : -1;
+      const int h = in ? g.hidx[v] : -1;
+      const bool both = in && find_node(me.b, B, v) >= 0;
+      const unsigned b_t = __ballot_sync(0xffffffffu, in && both && h >= 0);
+      const unsigned b_a = __ballot_sync(0xffffffffu, in && !both && h >= 0);
+      const unsigned b_l = __ballot_sync(0xffffffffu, in && h < 0);
+      x += __popc(__ballot_sync(0xffffffffu, both));
+      if (in && h >= 0) {
+        if (both) me.hub[2][nt + __popc(b_t & lt)] = h;
+        else me.hub[0][na + __popc(b_a & lt)] = h;
+        me.fa[q] = -1;
+      } else if (in) {
+        const int r = nl + __popc(b_l & lt);
+        me.list[r] = v;
+        me.fa[q] = (int8_t)r;
+      }
+      nt += __popc(b_t);
+      na += __popc(b_a);
+      nl += __popc(b_l);
+    }
+    for (int q0 = 0; q0 < B; q0 += 32) {
+      const int q = q0 + lane;
+      const bool in = q < B;
+      const int32_t v = in ? me.b[q] : -1;
+      const bool own = in && find_node(me.a, A, v) < 0;   // the others came with e_i
+      const int h = own ? g.hidx[v] : -1;
+      const unsigned b_b = __ballot_sync(0xffffffffu, own && h >= 0);
+      const unsigned b_l = __ballot_sync(0xffffffffu, own && h < 0);
+      if (own && h >= 0) {
+        me.hub[1][nb + __popc(b_b & lt)] = h;
+        me.fb[q] = -1;
+      } else if (own) {
+        const int r = nl + __popc(b_l & lt);
+        me.list[r] = v;
+        me.fb[q] = (int8_t)r;
+      }
+      nb += __popc(b_b);
+      nl += __popc(b_l);
+    }
+    __syncwarp();
+    auto code = [&](int C, int y, int z, int t) {
+      return (int)lut[ternary_code(A, B, C, x, y, z, t, theta)];
+    };
+    // the scan: steps [from, to) of all sizes
+    const int from = (int)((int64_t)n_steps * seg / g.n_seg);
+    const int to = na + nb + nt > 0 ? (int)((int64_t)n_steps * (seg + 1) / g.n_seg) : from;
+    int c = 0;
+    uint32_t bins[kOtfPop];
+#pragma unroll
+    for (int q = 0; q < kOtfPop; ++q) bins[q] = 0u;
+    for (int step = from; step < to; ++step) {
+      while (step >= s_step[c + 1]) ++c;
+      const int w = s_word[c] + (step - s_step[c]) * kOtfDrawWords + 4 * lane;
+      const bool in = w < s_word[c + 1];
+      uint32_t cnt[3][4][4];   // part, word, slice
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) cnt[p][r][q] = 0u;
+        const int nh = p == 0 ? na : p == 1 ? nb : nt;
+        for (int h0 = 0; h0 < nh; h0 += 4) {
+          uint4 v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            v[q] = in && h0 + q < nh
+                       ? __ldg((const uint4*)(g.pbits + (int64_t)me.hub[p][h0 + q] * g.Wp + w))
+                       : make_uint4(0u, 0u, 0u, 0u);
+          slice_add4(cnt[p][0][0], cnt[p][0][1], cnt[p][0][2], cnt[p][0][3], v[0].x, v[1].x,
+                     v[2].x, v[3].x);
+          slice_add4(cnt[p][1][0], cnt[p][1][1], cnt[p][1][2], cnt[p][1][3], v[0].y, v[1].y,
+                     v[2].y, v[3].y);
+          slice_add4(cnt[p][2][0], cnt[p][2][1], cnt[p][2][2], cnt[p][2][3], v[0].z, v[1].z,
+                     v[2].z, v[3].z);
+          slice_add4(cnt[p][3][0], cnt[p][3][1], cnt[p][3][2], cnt[p][3][3], v[0].w, v[1].w,
+                     v[2].w, v[3].w);
+        }
+      }
+      st_words += in ? 4 : 0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        uint32_t m[3][4];   // part -> ids with 0, 1, 2, 3 of its bitmap nodes
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+          const uint32_t c0 = cnt[p][r][0], c1 = cnt[p][r][1];
+          const uint32_t ge4 = cnt[p][r][2] | cnt[p][r][3];
+          m[p][0] = ~(c0 | c1 | ge4);
+          m[p][1] = c0 & ~(c1 | ge4);
+          m[p][2] = c1 & ~(c0 | ge4);
+          m[p][3] = c0 & c1 & ~ge4;
+        }
+        uint32_t rest = m[0][0] & m[1][0] & m[2][0];
+        int b = 0;
+#pragma unroll
+        for (int xt = 0; xt < 4; ++xt)
+#pragma unroll
+          for (int xb = 0; xb < 4 - xt; ++xb)
+#pragma unroll
+            for (int xa = 0; xa < 4 - xt - xb; ++xa) {
+              if (xa + xb + xt == 0) continue;
+              const uint32_t k = m[0][xa] & m[1][xb] & m[2][xt];
+              bins[b++] += __popc(k);
+              rest |= k;
+            }
+        // the others, a candidate a lane at a time (the loop is the warp's, or
+        // its lanes would part for good)
+        const uint32_t ov = cnt[0][r][3] | cnt[1][r][3] | cnt[2][r][3];
+        rest = ~(rest | ov);
+        while (__any_sync(0xffffffffu, rest != 0u)) {
+          const int bit = __ffs(rest) - 1;
+          if (rest) {
+            const int xa = sval(cnt[0][r][0], cnt[0][r][1], cnt[0][r][2], bit);
+            const int xb = sval(cnt[1][r][0], cnt[1][r][1], cnt[1][r][2], bit);
+            const int xt = sval(cnt[2][r][0], cnt[2][r][1], cnt[2][r][2], bit);
+            atomicAdd(&me.tab[xa + 8 * xb + 64 * xt], 1u);
+          }
+          rest &= rest - 1;
+        }
+        // a count of 8 or more: with every node at once
+        if (__any_sync(0xffffffffu, ov != 0u)) {
+          for (uint32_t todo = ov; todo; todo &= todo - 1) {
+            const int64_t k = g.id_of[(int64_t)(w + r) * 32 + __ffs(todo) - 1];
+            if (k == i || k == j) continue;
+            int z, y, t;
+            const int C = g.esize[k];
+            exact_overlaps(me.a, A, me.b, B, g.enode + g.eoff[k], C, z, y, t);
+            shared_bin_add(hist, code(C, y, z, t), 1);
+            ++st_cand;
+            ++st_exact;
+          }
+          __syncwarp();
+        }
+      }
+      if (step + 1 == to || step + 1 == s_step[c + 1]) {   // the end of this size
+        uint32_t v = 0u;
+#pragma unroll
+        for (int q = 0; q < kOtfPop; ++q) {
+          const uint32_t sum = __reduce_add_sync(0xffffffffu, bins[q]);
+          if (lane == q) v = sum;
+          bins[q] = 0u;
+        }
+        __syncwarp();
+        if (lane < kOtfPop) me.tab[kOtfPopKey[lane]] += v;
+        __syncwarp();
+        for (int q0 = 4 * lane; q0 < kOtfTab; q0 += 128) {
+          const uint4 v4 = *(const uint4*)&me.tab[q0];
+          if (!(v4.x | v4.y | v4.z | v4.w)) continue;
+          *(uint4*)&me.tab[q0] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const uint32_t num = u == 0 ? v4.x : u == 1 ? v4.y : u == 2 ? v4.z : v4.w;
+            if (!num) continue;
+            const int q = q0 + u, xa = q & 7, xb = (q >> 3) & 7, xt = q >> 6;
+            shared_bin_add(hist, code(c, xb + xt, xa + xt, xt), num);
+            st_cand += num;
+          }
+        }
+        __syncwarp();
+      }
+    }
+    // e_i and e_j were candidates of the scan
+    if (seg == 0 && lane < 2) {
+      const int xa = lane == 0 ? na : 0, xb = lane == 0 ? 0 : nb;
+      if (xa + xb + nt > 0 && xa < 8 && xb < 8 && nt < 8) {
+        shared_bin_add(hist, code(lane == 0 ? A : B, xb + nt, xa + nt, nt), -1);
+        --st_cand;
+      }
+    }
+    // list entries: each e_k at the first list node that it holds
+    for (int q = 0; q < nl; ++q) {
+      const int32_t v = me.list[q];
+      const int64_t end = g.voff[v + 1];
+      for (int64_t p = g.voff[v] + seg * 32 + lane; p < end; p += 32 * g.n_seg) {
+        const int64_t k = g.vedge[p];
+        ++st_ent;
+        if (k == i || k == j) continue;
+        const int64_t kb = g.eoff[k];
+        const int C = (int)(g.eoff[k + 1] - kb);
+        int y = 0, z = 0, t = 0, xa = 0, xb = 0, xt = 0, owner = kOtfNodes;
+        for (int s = 0; s < C; ++s) {
+          const int32_t u = g.enode[kb + s];
+          const int pa = find_node(me.a, A, u), pb = find_node(me.b, B, u);
+          if (pa < 0 && pb < 0) continue;
+          const int f = pa >= 0 ? me.fa[pa] : me.fb[pb];
+          z += pa >= 0;
+          y += pb >= 0;
+          t += pa >= 0 && pb >= 0;
+          if (f >= 0) {
+            owner = min(owner, f);
+          } else if (pa >= 0 && pb >= 0) {
+            ++xt;
+          } else if (pa >= 0) {
+            ++xa;
+          } else {
+            ++xb;
+          }
+        }
+        if (owner != q || xa >= 8 || xb >= 8 || xt >= 8) continue;
+        const int with = code(C, y, z, t);
+        if (xa + xb + xt == 0) {
+          shared_bin_add(hist, with, 1);
+          ++st_cand;
+        } else {
+          const int without = code(C, xb + xt, xa + xt, xt);
+          if (with != without) {
+            shared_bin_add(hist, without, -1);
+            shared_bin_add(hist, with, 1);
+          }
+        }
+      }
+    }
+    __syncwarp();
+  }
+  if (g.stats) {
+    for (int d = 16; d; d >>= 1) {
+      st_cand += __shfl_xor_sync(0xffffffffu, st_cand, d);
+      st_words += __shfl_xor_sync(0xffffffffu, st_words, d);
+      st_ent += __shfl_xor_sync(0xffffffffu, st_ent, d);
+      st_exact += __shfl_xor_sync(0xffffffffu, st_exact, d);
+    }
+    if (lane == 0) {
+      atomicAdd(&g.stats[0], st_cand);
+      atomicAdd(&g.stats[1], st_words);
+      atomicAdd(&g.stats[2], st_ent);
+      atomicAdd(&g.stats[3], st_exact);
+    }
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < 432; q += kOtfScanThreads)
+    if (hist[q]) atomicAdd(&g.hist[q], hist[q]);
+}
+
+// Hyperedges of each size (the counts are cleared before): 5, 11 and 30 us for
+// the three kernels that order 500,000 hyperedges by size.
+__global__ void k_otf_sizes(int64_t E, const uint8_t* __restrict__ esize, int32_t* counts) {
+  __shared__ int32_t s[kOtfSizes];
+  if (threadIdx.x < kOtfSizes) s[threadIdx.x] = 0;
+  __syncthreads();
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < E;
+       k += (int64_t)gridDim.x * blockDim.x)
+    atomicAdd(&s[esize[k]], 1);
+  __syncthreads();
+  if (threadIdx.x < kOtfSizes && s[threadIdx.x]) atomicAdd(&counts[threadIdx.x], s[threadIdx.x]);
+}
+
+// first word of each size, a multiple of four; counts -> next free position
+__global__ void k_otf_starts(int32_t* counts, int32_t* cls) {
+  if (threadIdx.x) return;
+  int32_t w = 0;
+  for (int c = 0; c < kOtfSizes; ++c) {
+    const int32_t n = counts[c];
+    cls[c] = w;
+    counts[c] = w * 32;
+    w += (n + 127) / 128 * 4;
+  }
+  cls[kOtfSizes] = w;
+}
+
+// position of each hyperedge in order of size (any order within a size)
+__global__ void k_otf_positions(int64_t E, const uint8_t* __restrict__ esize, int32_t* next,
+                                int32_t* __restrict__ pos_of, int32_t* __restrict__ id_of) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int c = k < E ? esize[k] : -1;
+  const unsigned peers = __match_any_sync(0xffffffffu, c);
+  if (c < 0) return;
+  const int lead = __ffs(peers) - 1;
+  int32_t at = 0;
+  if (lane == lead) at = atomicAdd(&next[c], __popc(peers));
+  at = __shfl_sync(peers, at, lead) + __popc(peers & ((1u << lane) - 1u));
+  pos_of[k] = at;
+  id_of[at] = (int32_t)k;
+}
+
+// membership bitmap of each bitmap node (its incidence list as bits); pbits
+// (may be null): the same in order of size
 __global__ void k_otf_bits(int64_t n_bitmaps, int64_t W, const int32_t* __restrict__ nodes_of,
                            const int64_t* __restrict__ voff, const int32_t* __restrict__ vedge,
-                           uint32_t* __restrict__ bits) {
+                           uint32_t* __restrict__ bits, int64_t Wp,
+                           const int32_t* __restrict__ pos_of, uint32_t* __restrict__ pbits) {
   for (int64_t h = blockIdx.x; h < n_bitmaps; h += gridDim.x) {
     const int32_t v = nodes_of[h];
     uint32_t* b = bits + h * W;
     for (int64_t q = voff[v] + threadIdx.x; q < voff[v + 1]; q += blockDim.x) {
       const int32_t e = vedge[q];
       atomicOr(&b[e >> 5], 1u << (e & 31));
+      if (pbits) {
+        const int32_t at = pos_of[e];
+        atomicOr(&pbits[h * Wp + (at >> 5)], 1u << (at & 31));
+      }
     }
   }
 }
@@ -702,6 +1242,11 @@ void release_onthefly(mochy_ctx* ctx) {
   ctx->otf_hbits = nullptr;
   ctx->otf_sbits = nullptr;
   ctx->otf_uprefix = nullptr;
+  ctx->otf_by_size = false;
+  ctx->otf_pbits = nullptr;
+  ctx->otf_id_of = ctx->otf_cls = nullptr;
+  ctx->otf_draws = nullptr;
+  ctx->otf_pwords = ctx->otf_max_draws = 0;
   ctx->otf_wedges = ctx->otf_bitmaps = ctx->otf_words = 0;
 }
 
@@ -734,11 +1279,24 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
   auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t b_hidx = al((size_t)std::max<int64_t>(N, 1) * 4);
   const size_t b_nodes = al(nodes_of.size() * 4);
-  const size_t b_bits = al((size_t)std::max<int64_t>(max_bitmaps, 1) * W * 4);
+  // bitmaps in order of size as well when all of both fit the budget; each of
+  // the 64 sizes begins on four words
+  const int64_t Wp = W + 4 * kOtfSizes;
+  const bool by_size = max_bitmaps == (int64_t)pop.size() &&
+                       (int64_t)pop.size() * (W + Wp) * 4 <= cap_bytes;
+  const size_t b_one = al((size_t)std::max<int64_t>(max_bitmaps, 1) * W * 4);
+  const size_t b_bits = by_size ? b_one + al((size_t)std::max<int64_t>(max_bitmaps, 1) * Wp * 4)
+                                : b_one;
   const size_t b_sbits = al((size_t)4 * W * 4);
   const size_t b_pre = al((size_t)(E + 1) * 8);
-  const size_t b_deg = al((size_t)std::max<int64_t>(E, 1) * 8);
-  const size_t bytes = b_hidx + b_nodes + b_bits + b_sbits + b_pre + 2 * b_deg;
+  // by size: the positions (both ways) and the sizes' first words take the
+  // place of the degrees, and the draws of a launch that of the neighbours
+  // after i, once these are summed
+  const size_t b_pos = al((size_t)std::max<int64_t>(E, 1) * 4), b_id = al((size_t)Wp * 32 * 4);
+  const size_t b_deg = by_size ? b_pos + b_id + al((2 * kOtfSizes + 1) * 4)
+                               : al((size_t)std::max<int64_t>(E, 1) * 8);
+  const size_t b_up = std::max(al((size_t)std::max<int64_t>(E, 1) * 8), kOtfDrawBytes);
+  const size_t bytes = b_hidx + b_nodes + b_bits + b_sbits + b_pre + b_deg + b_up;
   void* p = nullptr;
   MOCHY_TRY(dev_alloc(ctx, &p, bytes));
   char* c = (char*)p;
@@ -758,12 +1316,35 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
                       st) != cudaSuccess ||
       cudaMemsetAsync(ctx->otf_hbits, 0, b_bits + b_sbits, st) != cudaSuccess)
     return bail(fail(MOCHY_E_CUDA, "on-the-fly set-up copy failed"));
+  ctx->otf_by_size = by_size;
+  if (by_size) {
+    ctx->otf_pwords = Wp;
+    ctx->otf_pbits = (uint32_t*)((char*)ctx->otf_hbits + b_one);
+    ctx->otf_id_of = (int32_t*)((char*)deg + b_pos);
+    ctx->otf_cls = (int32_t*)((char*)deg + b_pos + b_id);
+    ctx->otf_draws = up;
+    ctx->otf_max_draws = (int64_t)(b_up / 8);
+    int32_t* counts = ctx->otf_cls + kOtfSizes + 1;
+    if (cudaMemsetAsync(counts, 0, kOtfSizes * 4, st) != cudaSuccess)
+      return bail(fail(MOCHY_E_CUDA, "on-the-fly set-up copy failed"));
+    if (E > 0) {
+      k_otf_sizes<<<(unsigned)std::min<int64_t>(ceil_div(E, 256), (int64_t)ctx->num_sms * 4), 256, 0,
+                    st>>>(E, ctx->esize, counts);
+      k_otf_starts<<<1, 32, 0, st>>>(counts, ctx->otf_cls);
+      k_otf_positions<<<(unsigned)ceil_div(E, 256), 256, 0, st>>>(E, ctx->esize, counts,
+                                                                 (int32_t*)deg, ctx->otf_id_of);
+      note_launch();
+      note_launch();
+      note_launch();
+    }
+  }
   if (max_bitmaps > 0) {
     k_otf_bits<<<(unsigned)std::min<int64_t>(max_bitmaps, 4096), 256, 0, st>>>(
-        max_bitmaps, W, d_nodes_of, ctx->voff, ctx->vedge, ctx->otf_hbits);
+        max_bitmaps, W, d_nodes_of, ctx->voff, ctx->vedge, ctx->otf_hbits, Wp, (int32_t*)deg,
+        by_size ? ctx->otf_pbits : nullptr);
     note_launch();
   }
-  if (E > 0) {
+  if (E > 0 && !by_size) {
     k_otf_size_bits<<<ceil_div(E, 256), 256, 0, st>>>(E, W, ctx->esize, ctx->otf_sbits);
     note_launch();
   }
@@ -847,6 +1428,37 @@ int count_sampled_onthefly(mochy_ctx* ctx, int64_t samples, uint64_t seed, int64
   g.queue = ctx->counters + 4;   // 64-bit counter over words 4 and 5
   g.stats = d_stats;
   if (d_stats) MOCHY_CUDA(cudaMemsetAsync(d_stats, 0, 4 * 8, st));
+  if (ctx->otf_by_size) {
+    g.Wp = ctx->otf_pwords;
+    g.pbits = ctx->otf_pbits;
+    g.cls = ctx->otf_cls;
+    g.id_of = ctx->otf_id_of;
+    g.draws = (int2*)ctx->otf_draws;
+    int per_sm = 0;
+    MOCHY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_otf_classify,
+                                                             kOtfScanThreads, 0));
+    const int64_t warps = (int64_t)ctx->num_sms * std::max(per_sm, 1) * (kOtfScanThreads / 32);
+    const int64_t steps = std::max<int64_t>(g.W / kOtfDrawWords, 1);
+    for (int64_t first = 0; first < samples; first += ctx->otf_max_draws) {
+      g.first = first;
+      g.n_draws = std::min(samples - first, ctx->otf_max_draws);
+      // a scan is cut when there are fewer than kOtfItems draws to a warp,
+      // into parts of kOtfMinSteps steps at least
+      g.n_seg = std::max<int64_t>(
+          1, std::min((kOtfItems * warps + g.n_draws - 1) / g.n_draws, steps / kOtfMinSteps));
+      if (first > 0) MOCHY_CUDA(cudaMemsetAsync(g.queue, 0, 8, st));
+      k_otf_draw<<<(unsigned)std::min<int64_t>(ceil_div(g.n_draws, kOtfScanThreads / 32),
+                                               (int64_t)ctx->num_sms * 8),
+                   kOtfScanThreads, 0, st>>>(g);
+      k_otf_classify<<<(unsigned)std::min<int64_t>(
+                           ceil_div(g.n_draws * g.n_seg, kOtfScanThreads / 32),
+                           (int64_t)ctx->num_sms * std::max(per_sm, 1)),
+                       kOtfScanThreads, 0, st>>>(g);
+      note_launch();
+      MOCHY_LAUNCHED();
+    }
+    return MOCHY_OK;
+  }
   const size_t smem = otf_smem_bytes();
   MOCHY_TRY(ensure_dynamic_smem((const void*)k_otf_sample, smem));
   int per_sm = 0;

@@ -463,7 +463,10 @@ void* mochy_stream(mochy_ctx* ctx);
 int mochy_trace(mochy_ctx* ctx, int level);
 int mochy_trace_read(mochy_ctx* ctx, char* buf, int64_t len);
 
-/* Bytes of device memory the context holds now. */
+/* Bytes of device memory the context holds now.  Not counted are the blocks
+ * that it has given up and keeps for its next allocations: at most 16 GB and
+ * 64 blocks, within hbm_budget_bytes where one is set, given back when an
+ * allocation of any context on the device would fail, and by mochy_destroy. */
 int64_t mochy_device_bytes(mochy_ctx* ctx);
 
 /* Number of kernels the library launched in this process (for accounting). */

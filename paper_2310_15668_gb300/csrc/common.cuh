@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/mochy.h"
@@ -90,6 +91,13 @@ struct Buffer {
 }  // namespace mochy
 
 struct mochy_ctx {
+  // device blocks given up by this context and kept for its next allocations
+  // (api.cu); kept_max = 0: none are kept
+  struct Kept { void* p; size_t bytes; };
+  std::vector<Kept> kept;
+  std::unordered_map<void*, size_t> capacity;   // blocks in use that are larger than asked for
+  size_t kept_bytes = 0, kept_max = 0;
+  mochy_ctx* copies = nullptr;                  // mochy_profile's randomized copies
   int device = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;

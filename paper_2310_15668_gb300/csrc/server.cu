@@ -29,6 +29,7 @@ namespace mochy {
 int64_t estimate_graph_bytes(int64_t n_nodes, int64_t n_edges, const int64_t* off,
                              const int32_t* nodes);   // batch.cu
 void release_scratch(mochy_ctx* ctx);                 // api.cu
+void keep_no_blocks(mochy_ctx* ctx);                  // api.cu
 
 namespace {
 
@@ -149,6 +150,7 @@ void worker_main(mochy_server* s) {
     s->cv_done.notify_all();
     return;
   }
+  keep_no_blocks(ctx);           // a request's memory is given back at its end
   for (;;) {
     std::unique_ptr<Request> r;
     {

@@ -75,6 +75,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_partials_scan(int64_t* pa
   }
 }
 
+// Each block scans its tile from what lies before it: with kSum the sum of the
+// partials before its own (nb of at most kScanThreads), else partial[blockIdx],
+// already scanned.  One tile alone (partial null) starts at 0.
+template <bool kSum>
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int64_t* __restrict__ in, int64_t n,
                              const int64_t* __restrict__ partial, int64_t* __restrict__ out) {
   const int64_t tile = (int64_t)blockIdx.x * kScanTile;
@@ -86,8 +90,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int64_t* __re
     v[r] = i < n ? in[i] : 0;
     s += v[r];
   }
-  int64_t total;
-  int64_t ex = block_excl_scan(s, &total) + partial[blockIdx.x];
+  int64_t total, before = 0;
+  if (kSum) {
+    if (partial)
+      block_excl_scan(threadIdx.x < blockIdx.x ? partial[threadIdx.x] : 0, &before);
+  } else {
+    before = partial[blockIdx.x];
+  }
+  int64_t ex = block_excl_scan(s, &total) + before;
 #pragma unroll
   for (int r = 0; r < kScanItems; ++r) {
     int64_t i = tile + (int64_t)threadIdx.x * kScanItems + r;
@@ -168,17 +178,31 @@ int bits_for(int64_t n) {
   return b;
 }
 
+// Launches bound a scan of less than a few million values (2.5 to 4 us each,
+// and a call that loads, projects and counts has nine or more): one for a
+// single tile of 4,096, two where a block can add the partials before it
+// itself (4.2 million), else three.
 int scan_exclusive_i64(mochy_ctx* ctx, const int64_t* d_in, int64_t* d_out, int64_t n) {
   if (n <= 0) return MOCHY_OK;
   const int64_t nb = (n + kScanTile - 1) / kScanTile;
+  if (nb == 1) {
+    k_scan_apply<true><<<1, kScanThreads, 0, ctx->stream>>>(d_in, n, nullptr, d_out);
+    MOCHY_LAUNCHED();
+    return MOCHY_OK;
+  }
   void* part = nullptr;
   MOCHY_TRY(scratch(ctx, 3, sizeof(int64_t) * (size_t)nb, &part));
   int64_t* partial = (int64_t*)part;
   k_scan_partials<<<(unsigned)nb, kScanThreads, 0, ctx->stream>>>(d_in, n, partial);
   MOCHY_LAUNCHED();
+  if (nb <= kScanThreads) {
+    k_scan_apply<true><<<(unsigned)nb, kScanThreads, 0, ctx->stream>>>(d_in, n, partial, d_out);
+    MOCHY_LAUNCHED();
+    return MOCHY_OK;
+  }
   k_scan_partials_scan<<<1, kScanThreads, 0, ctx->stream>>>(partial, nb);
   MOCHY_LAUNCHED();
-  k_scan_apply<<<(unsigned)nb, kScanThreads, 0, ctx->stream>>>(d_in, n, partial, d_out);
+  k_scan_apply<false><<<(unsigned)nb, kScanThreads, 0, ctx->stream>>>(d_in, n, partial, d_out);
   MOCHY_LAUNCHED();
   return MOCHY_OK;
 }

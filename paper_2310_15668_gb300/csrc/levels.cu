@@ -42,6 +42,19 @@
 // every region state stays the same), and one last kernel turns the tables
 // into motif counts.  On the Zipf hypergraphs of the benchmark 1.5 to 4 % of
 // the closed instances have three heavy pairs.
+//
+// Measured (Zipf(1.0) members, sizes s^-2.5 on [2, 25]), 10,000 / 60,000
+// hyperedges, each kernel alone, and what bounds it:
+//   k_lv_fill         0.12 /  2.1 ms  reads the line graph once (HBM at 60,000)
+//   k_lv_triples      0.54 / 23   ms  L1 sectors of the overlap matrix, latency
+//   k_lv_many         0.56 /  8.9 ms  shared-memory multiply-adds of class pairs
+//   k_lv_light        0.30 /  4.6 ms  gathers of hyperedges at unpopular nodes
+//   k_lv_open         0.15 /  1.0 ms  shared atomics
+//   k_lv_tri          0.21 /  0.95 ms gathers of node-pair counts
+//   k_lv_few          0.12 /  0.25 ms hash probes
+//   k_lv_light_pairs  0.10 /  0.28 ms the same
+// They run side by side on four streams: a whole count 1.3 / 31 ms, against
+// 21 / 890 ms for the triangle kernels of count_split.cu.
 #include <cstring>
 
 #include "classify.cuh"
@@ -68,7 +81,9 @@ struct LevelUnit {
   int64_t hmoff;    // first entry of its hub matrix
 };
 
-constexpr int kFewHeavy = 16;   // level 2: centres of at most this many heavy pairs, pair by pair
+// Level 2: centres of at most this many heavy pairs go pair by pair (8 and 32:
+// within 5 % of 16 at 2,000 to 60,000 hyperedges).
+constexpr int kFewHeavy = 16;
 
 constexpr int kMaxHubs = 4096;   // hubs of one unit (their pair counts are a matrix)
 
@@ -1638,76 +1653,143 @@ k_lv_open(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, int 
 // Tables to motif counts
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256)
-k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, int n_bins) {
-  extern __shared__ unsigned long long hist[];
-  const int unit = blockIdx.y, Q = g.Q;
-  for (int q = threadIdx.x; q < n_bins; q += blockDim.x) hist[q] = 0ull;
+// An entry costs up to 60 adds to few and popular bins, and most entries are 0.
+// So a block first queues the non-zero entries of its chunk, then gives the
+// parts of each (one add_closed, at most kParts) to threads of their own, and
+// the lanes of a warp add to copies of the histogram.
+// Shared atomics on equal bins bound it: 55 -> 43 us at 2,000 hyperedges, 96 ->
+// 61 us at 7,001 with theta = 2, 920 -> 300 us for a batch of 54 (a thread an
+// entry and one histogram a block before; a call of add_closed for each part at
+// a place of its own, where the lanes part, took 350 us at 2,000).
+constexpr int kFinishThreads = 256;
+constexpr int kFinishChunk = 2048;   // entries of a block, at most
+constexpr int kFinishCopies = 8;
+constexpr int kParts = 16;
+
+// One add_closed.  The parts are selected into it and added at one place, so
+// that the lanes of a warp add together.
+struct Part {
+  int A, B, C, x, y, z, t;
+  long long n;
+};
+
+// part p of an instance of three heavy pairs: itself (0), what the levels 1
+// and 2 count for it from centre (p - 1) / 4, and what level 0 does (13, 14)
+__device__ __forceinline__ Part triple_part(int p, int A, int B, int C, int x, int y, int z, int t,
+                                            long long n) {
+  Part o = {A, B, C, x, y, z, t, p == 0 ? n : 0};
+  if (p >= 13) o = {A, B, C, 1, 1, 1, p == 13 ? 1 : 0, p == 13 ? -n * t : 0};
+  long long ft = -((long long)x * y * z - (long long)t * (x + y + z) + 2 * t);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    // centre A with pairs (A, B) of overlap x and (A, C) of z; opposite y
+    const long long out =
+        -(long long)(y - t) * (z - t) + (long long)(y - t) * z + (long long)(z - t) * y;
+    const int k = p - 1 - 4 * i;
+    if (k >= 0 && k < 4)
+      o = {A, B, C, x, 1, k < 2 ? z : 1, k & 1 ? 0 : 1,
+           k == 0 ? -n * t : k == 1 ? -n * (y - t) : k == 2 ? n * t : n * out};
+    ft += (long long)t * (x - 1) * (z - 1) + (long long)(y - t) * x * z - out * x;
+    // rotate: A -> B -> C -> A
+    const int ta = A, tx = x;
+    A = B; B = C; C = ta;
+    x = y; y = z; z = tx;
+  }
+  if (p == 14) o.n = n * ft;
+  return o;
+}
+
+__device__ __forceinline__ Part entry_part(const LevelArgs& g, int64_t at, int part, long long n) {
+  const int Q = g.Q;
+  if (at >= g.o_trip) {
+    int e = (int)(at - g.o_trip), t = kTripleT - 1;
+    while (e < g.tt.off[t]) --t;
+    e -= g.tt.off[t];
+    const int m = g.tt.n[t], lo = g.tt.lo[t], c = t + g.theta + 2;
+    const int c1 = e % c, b1 = e / c % c, a1 = e / (c * c) % c;
+    e /= c * c * c;
+    const int r = e % m + lo, q = e / m % m + lo, p = e / (m * m) + lo;
+    const int x = t + p, y = t + q, z = t + r;
+    return triple_part(part, a1 + x + r, b1 + x + q, c1 + y + r, x, y, z, t, n);
+  }
+  if (at >= g.o_in2) {
+    const bool inside = at < g.o_out2;
+    const int64_t e = at - (inside ? g.o_in2 : g.o_out2);
+    int A = 2;
+    while (A < g.S && e >= level2_at(A + 1, Q)) ++A;
+    const int ncl = (A - 1) * Q;
+    const int r = (int)(e - level2_at(A, Q));
+    const int i = r / ncl, j = r - i * ncl;
+    const int x = i / Q + 2, z = j / Q + 2, B = x + i % Q, C = z + j % Q;
+    const int t = inside ? 1 : 0;
+    if (part == 0) return {A, B, C, x, 1, z, t, n};
+    if (part == 1) return {A, B, C, x, 1, 1, t, inside ? -n : -n * z};
+    if (part == 2) return {A, C, B, z, 1, 1, t, inside ? -n : -n * x};
+    if (part == 3) return {A, B, C, 1, 1, 1, t, inside ? n : n * x * z};
+    return {A, B, C, 1, 1, 1, 0, part == 4 && inside ? -n * (x - 1) * (z - 1) : 0};
+  }
+  if (at >= g.o_in1) {
+    const bool inside = at < g.o_out1;
+    const int e = (int)(at - (inside ? g.o_in1 : g.o_out1));
+    const int C = e % Q + 1, dB = e / Q % Q, dA = e / (Q * Q) % Q, x = e / (Q * Q * Q) + 2;
+    const long long half = n / 2;   // each pair was met from both of its rows
+    const int t = inside ? 1 : 0;
+    if (part == 0) return {x + dA, x + dB, C, x, 1, 1, t, half};
+    return {x + dA, x + dB, C, 1, 1, 1, t, part > 1 ? 0 : inside ? -half : -half * x};
+  }
+  const bool star = at < g.o_tri;
+  const int e = (int)(at - (star ? g.o_star : g.o_tri));
+  return {e / (Q * Q) + 1, e / Q % Q + 1, e % Q + 1, 1, 1, 1, star ? 1 : 0, part == 0 ? n : 0};
+}
+
+__global__ void __launch_bounds__(kFinishThreads)
+k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, int n_bins,
+            int chunk, int copies) {
+  extern __shared__ unsigned long long hists[];   // [copies][n_bins + 1]
+  __shared__ int32_t queue[kFinishChunk];
+  __shared__ int32_t n_queue;
+  const int unit = blockIdx.y;
+  unsigned long long* hist = hists + (threadIdx.x & (copies - 1)) * (n_bins + 1);
+  for (int q = threadIdx.x; q < copies * (n_bins + 1); q += kFinishThreads) hists[q] = 0ull;
+  if (threadIdx.x == 0) n_queue = 0;
   __syncthreads();
   const int64_t* tab = g.tab + unit * g.tab_stride;
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; at < g.n_tab; at += step) {
-    const long long n = tab[at];
-    if (!n) continue;
-    if (at >= g.o_trip) {
-      int e = (int)(at - g.o_trip), t = kTripleT - 1;
-      while (e < g.tt.off[t]) --t;
-      e -= g.tt.off[t];
-      const int m = g.tt.n[t], lo = g.tt.lo[t], c = t + g.theta + 2;
-      const int c1 = e % c, b1 = e / c % c, a1 = e / (c * c) % c;
-      e /= c * c * c;
-      const int r = e % m + lo, q = e / m % m + lo, p = e / (m * m) + lo;
-      const int x = t + p, y = t + q, z = t + r;
-      add_triple(hist, cd, a1 + x + r, b1 + x + q, c1 + y + r, x, y, z, t, n);
-    } else if (at >= g.o_in2) {
-      const bool inside = at < g.o_out2;
-      const int64_t e = at - (inside ? g.o_in2 : g.o_out2);
-      int A = 2;
-      while (A < g.S && e >= level2_at(A + 1, Q)) ++A;
-      const int ncl = (A - 1) * Q;
-      const int r = (int)(e - level2_at(A, Q));
-      const int i = r / ncl, j = r - i * ncl;
-      const int x = i / Q + 2, z = j / Q + 2, B = x + i % Q, C = z + j % Q;
-      if (inside) {
-        add_closed(hist, cd, A, B, C, x, 1, z, 1, n);
-        add_closed(hist, cd, A, B, C, x, 1, 1, 1, -n);
-        add_closed(hist, cd, A, C, B, z, 1, 1, 1, -n);
-        add_closed(hist, cd, A, B, C, 1, 1, 1, 1, n);
-        add_closed(hist, cd, A, B, C, 1, 1, 1, 0, -n * (x - 1) * (z - 1));
-      } else {
-        add_closed(hist, cd, A, B, C, x, 1, z, 0, n);
-        add_closed(hist, cd, A, B, C, x, 1, 1, 0, -n * z);
-        add_closed(hist, cd, A, C, B, z, 1, 1, 0, -n * x);
-        add_closed(hist, cd, A, B, C, 1, 1, 1, 0, n * x * z);
-      }
-    } else if (at >= g.o_in1) {
-      const bool inside = at < g.o_out1;
-      int e = (int)(at - (inside ? g.o_in1 : g.o_out1));
-      const int C = e % Q + 1, dB = e / Q % Q, dA = e / (Q * Q) % Q, x = e / (Q * Q * Q) + 2;
-      const long long half = n / 2;   // each pair was met from both of its rows
-      add_closed(hist, cd, x + dA, x + dB, C, x, 1, 1, inside ? 1 : 0, half);
-      add_closed(hist, cd, x + dA, x + dB, C, 1, 1, 1, inside ? 1 : 0, inside ? -half : -half * x);
-    } else {
-      const bool star = at < g.o_tri;
-      const int e = (int)(at - (star ? g.o_star : g.o_tri));
-      add_closed(hist, cd, e / (Q * Q) + 1, e / Q % Q + 1, e % Q + 1, 1, 1, 1, star ? 1 : 0, n);
-    }
+  const int64_t first = (int64_t)blockIdx.x * chunk;
+  for (int q = threadIdx.x; q < chunk && first + q < g.n_tab; q += kFinishThreads)
+    if (tab[first + q]) queue[atomicAdd(&n_queue, 1)] = q;
+  __syncthreads();
+  for (int w = threadIdx.x; w < n_queue * kParts; w += kFinishThreads) {
+    const int64_t at = first + queue[w / kParts];
+    const Part o = entry_part(g, at, w % kParts, tab[at]);
+    add_closed(hist, cd, o.A, o.B, o.C, o.x, o.y, o.z, o.t, o.n);
   }
   // the tuples outside the table
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s <= (int64_t)g.omask; s += step) {
-    unsigned long long k = g.okey[s];
-    if (!k) continue;
-    --k;
-    const int c1 = (int)(k & 127), b1 = (int)(k >> 7 & 127), a1 = (int)(k >> 14 & 127);
-    const int r = (int)(k >> 21 & 63), q = (int)(k >> 27 & 63), p = (int)(k >> 33 & 63),
-              t = (int)(k >> 39 & 63);
-    if ((int)(k >> 45) != unit) continue;
-    const int x = t + p, y = t + q, z = t + r;
-    add_triple(hist, cd, a1 + x + r, b1 + x + q, c1 + y + r, x, y, z, t, (long long)g.ocnt[s]);
+  for (int64_t s0 = (int64_t)blockIdx.x * kFinishThreads; s0 <= (int64_t)g.omask;
+       s0 += (int64_t)gridDim.x * kFinishThreads) {
+    __syncthreads();
+    if (threadIdx.x == 0) n_queue = 0;
+    __syncthreads();
+    const unsigned long long k = g.okey[s0 + threadIdx.x];   // slots: a multiple of the threads
+    if (k && (int)((k - 1) >> 45) == unit) queue[atomicAdd(&n_queue, 1)] = threadIdx.x;
+    __syncthreads();
+    for (int w = threadIdx.x; w < n_queue * kParts; w += kFinishThreads) {
+      const int64_t s = s0 + queue[w / kParts];
+      const unsigned long long e = g.okey[s] - 1;
+      const int c1 = (int)(e & 127), b1 = (int)(e >> 7 & 127), a1 = (int)(e >> 14 & 127);
+      const int r = (int)(e >> 21 & 63), q = (int)(e >> 27 & 63), p = (int)(e >> 33 & 63),
+                t = (int)(e >> 39 & 63);
+      const int x = t + p, y = t + q, z = t + r;
+      const Part o = triple_part(w % kParts, a1 + x + r, b1 + x + q, c1 + y + r, x, y, z, t,
+                                 (long long)g.ocnt[s]);
+      add_closed(hist, cd, o.A, o.B, o.C, o.x, o.y, o.z, o.t, o.n);
+    }
   }
   __syncthreads();
-  for (int q = threadIdx.x; q < n_bins; q += blockDim.x)
-    if (hist[q]) atomicAdd(&hist_out[(int64_t)unit * n_bins + q], hist[q]);
+  for (int q = threadIdx.x; q < n_bins; q += kFinishThreads) {
+    unsigned long long v = 0ull;
+    for (int c = 0; c < copies; ++c) v += hists[c * (n_bins + 1) + q];
+    if (v) atomicAdd(&hist_out[(int64_t)unit * n_bins + q], v);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1717,6 +1799,9 @@ k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, in
 // Largest theta (or kh threshold) counted by levels: the table of level 3
 // must fit shared memory.
 constexpr int kMaxTheta = 4;
+// Nodes in this many hyperedges are hubs, whose node pairs are a matrix; the
+// others' are read from their hyperedges (16: 49 ms at 60,000 hyperedges, 64:
+// 3.46 ms at 10,000, against 44 and 2.84).
 constexpr int kHubDeg = 32;
 
 // table of tuples for a threshold, with the usual ranges of p, q, r
@@ -2028,10 +2113,14 @@ int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const 
   MOCHY_LAUNCHED();
   MOCHY_TRY(join_sides(ctx, kSides));
   if (timer) timer->mark("level 3");
-  const int64_t want = ceil_div(std::max<int64_t>(g.n_tab, (int64_t)g.omask + 1), 256);
-  k_lv_finish<<<dim3((unsigned)std::max<int64_t>(8, std::min<int64_t>(want, ctx->num_sms * 8 / g.n_units)),
-                     g.n_units), 256, (size_t)n_bins * 8, st>>>(
-      g, cd, d_hist, n_bins);
+  // chunks of one entry a thread while all blocks fit four waves
+  int chunk = kFinishThreads, copies = kFinishCopies;
+  while (chunk < kFinishChunk &&
+         ceil_div(g.n_tab, chunk) * (int64_t)g.n_units > (int64_t)ctx->num_sms * 32)
+    chunk *= 2;
+  while (copies > 1 && (size_t)copies * (n_bins + 1) * 8 > 32 * 1024) copies /= 2;
+  k_lv_finish<<<dim3((unsigned)ceil_div(g.n_tab, chunk), g.n_units), kFinishThreads,
+                (size_t)copies * (n_bins + 1) * 8, st>>>(g, cd, d_hist, n_bins, chunk, copies);
   MOCHY_LAUNCHED();
   if (timer) timer->mark("finish");
   return MOCHY_OK;

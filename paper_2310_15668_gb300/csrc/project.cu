@@ -11,6 +11,10 @@
 // degree have their list as a bitmap too, so that the first step costs them
 // one word per 32 ids; rows without such a node skip the chunks that none of
 // their lists reaches.
+// Issue and shared-memory latency bound it (4.7 warp instructions an entry, 42 %
+// of the issue slots, 20 warps an SM): 100,001 Zipf(1.0) hyperedges, 9.9 GB of
+// line graph, 13.3 ms for both passes, against 56 for windows of list entries;
+// 4 or 6 blocks an SM instead of 8: 21 and 18 ms, blocks of 256 threads 19.
 #include "common.cuh"
 
 namespace mochy {
@@ -22,8 +26,9 @@ constexpr int kChunkBits = 10;                   // ids per chunk: one word a la
 constexpr int kChunk = 1 << kChunkBits;
 
 // A node gets a bitmap when it lies in at least this many hyperedges of its
-// unit: four or more per chunk, so that its words are worth reading.  The
-// bitmaps then take at most 9 words per incidence.
+// unit: four or more per chunk, so that its words are worth reading (a 128th
+// and a 512th instead of a 256th: within 2 % at 10,000 and 100,001
+// hyperedges).  The bitmaps then take at most 9 words per incidence.
 __device__ __forceinline__ int64_t bitmap_degree(int64_t unit_edges) {
   return max((int64_t)32, unit_edges >> 8);
 }

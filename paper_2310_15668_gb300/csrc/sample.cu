@@ -740,18 +740,25 @@ __global__ void __launch_bounds__(kPlusThreads, 2) k_sample_pairs(RowsArgs r) {
 
 size_t rows_smem_bytes(int64_t n_edges) { return (size_t)((n_edges + 7) / 8) * 4; }
 
-// Rows this long are streamed (k_sample_rows): the block's barriers per work
+// Average degrees from which rows are streamed: the block's barriers per work
 // item cost about as much as merging rows of a few hundred entries by a warp.
-constexpr int64_t kRowsMinDegree = 256;
+// Streamed / merged at average degree 124, 174, 246, 369, 2,507: A+ (20,000
+// draws; 4,000 at the last) 0.34 / 0.14, 0.32 / 0.18, 0.32 / 0.24, 0.33 / 0.35,
+// 0.24 / 0.48 ms; A (300 draws; 80) 0.24 / 0.19, 0.29 / 0.31, 0.32 / 0.53,
+// 0.47 / 1.23, 2.1 / 10.4 ms.
+constexpr int64_t kPlusMinDegree = 256, kRowsMinDegree = 160;
 
-// draws from which they are sorted by row (about 80 us of small launches)
+// Draws from which they are sorted by row: the small launches take about 30 us
+// (1,000 and 4,000 draws: 0.165 and 0.273 ms sorted, 0.132 and 0.241 not;
+// 16,000: 0.58 and 0.70).
 constexpr int64_t kGroupDraws = 4096;
 
 // work items per hyperedge from which MoCHy-A makes the class histograms
 constexpr int64_t kClassesFrom = 1;
 
-bool use_rows(const mochy_ctx* ctx) {
-  return ctx->theta <= kRowsMaxTheta && ctx->n_wedges * 2 >= kRowsMinDegree * ctx->n_edges &&
+bool use_rows(const mochy_ctx* ctx, int method) {
+  const int64_t degree = method == MOCHY_A_PLUS ? kPlusMinDegree : kRowsMinDegree;
+  return ctx->theta <= kRowsMaxTheta && ctx->n_wedges * 2 >= degree * ctx->n_edges &&
          rows_smem_bytes(ctx->n_edges) + 50 * 1024 <= ctx->smem_optin;
 }
 
@@ -822,7 +829,7 @@ int count_sampled(mochy_ctx* ctx, int method, int64_t samples, uint64_t seed,
     g.sample_row = row;
   }
   if (n_items == 0) return MOCHY_OK;
-  if (use_rows(ctx) && samples <= 0xffffffffll &&
+  if (use_rows(ctx, method) && samples <= 0xffffffffll &&
       (method == MOCHY_A_PLUS || n_items >= kClassesFrom * ctx->n_edges)) {
     RowsArgs r{};
     r.g = g;

@@ -13,8 +13,10 @@ by the step time.
 value: inputs already resident in device memory, CUDA events on the
 library's stream around K steps.  e2e: the same metric through mochy_load
 from pinned host buffers (host-to-device copy inside the timed region) and a
-device-to-host read of the counts.  roofline: the dominant kernel's duration
-is taken live from the library's traced CUDA events.  cpu_baseline: the
+device-to-host read of the counts.  roofline: the line graph's bytes over the
+duration of the dominant phase, taken live from the library's traced CUDA
+events.  trace: the statistics of one more, untimed step through the kernels
+that classify candidate by candidate (trace level 2).  cpu_baseline: the
 CPU oracle (its anchor loop on every host core) on a seeded anchor sample of
 the same hypergraph.  sampled: candidates classified/s of MoCHy-A+ with
 r = 2,000,000 hyperwedges on the same projected hypergraph.  onthefly (rank
@@ -60,14 +62,6 @@ UNIT = "triples/s"
 
 
 WORKLOADS = ("medium", "tiny", "zipf10k", "zipf40k")
-
-# DRAM bytes (read + write) of one k_dense_triangles launch, measured with
-# ncu (dram__bytes_read.sum + dram__bytes_write.sum, one pass) on the
-# workload and threshold named, for the kernel as it is now; reported as
-# null for any other workload or threshold, and emptied whenever the kernel
-# changes until it is measured again.
-DENSE_TRAFFIC = {("medium", 1024): 8.640e12}
-
 
 def _spec(workload: str, seed_offset: int):
     """The bench workload (medium) or a smaller case of the same shape for
@@ -506,16 +500,16 @@ def run_gpu(args):
     d_nodes = torch.from_numpy(nodes).cuda()
     ctx = B.Context(device=local, dense_threshold=args.dense_threshold)
     stream = torch.cuda.ExternalStream(ctx.stream, device=local)
-    instances = 0
+    instances = n_wedges = 0
 
     shard = args.shard_rows and ws > 1
     my_rows = None
 
     def step(trace=False):
-        nonlocal instances, my_rows
+        nonlocal instances, my_rows, n_wedges
         B.mochy_load_device(ctx.h, spec.n_nodes, off.size - 1, d_off.data_ptr(),
                             d_nodes.data_ptr())
-        ctx.project()
+        n_wedges = ctx.project()[0]
         if shard:
             # one hypergraph, rows dealt to ranks; the share of each rank's
             # rows summed over ranks is the exact count
@@ -556,7 +550,8 @@ def run_gpu(args):
     ms_max, total_units = reduce_over_ranks(ms, units_here, ws, "cuda")
     value = total_units / (ms_max / 1000.0)
 
-    # kernel statistics (scanned words) from one more, untimed step at trace level 2
+    # statistics of the candidate-by-candidate kernels, from one more, untimed step
+    # at trace level 2 (which selects them)
     B.mochy_trace(ctx.h, 2)
     step()
     stats_trace = B.mochy_trace_read(ctx.h)
@@ -586,37 +581,24 @@ def run_gpu(args):
     if rank != 0:
         ctx.close()
         return 0
-    # roofline of the dominant kernel, from the traced events of the timed steps
+    # roofline of the dominant phase, from the traced events of the timed steps
     peak, peak_kind = _peaks()
     keys = set().union(*(p["phases_ms"].keys() for p in phases)) if phases else set()
     avg = {k: float(np.mean([p["phases_ms"].get(k, 0.0) for p in phases])) for k in keys}
     dom = max(avg, key=avg.get) if avg else None
     st = stats_trace
     roof = None
-    if dom == "dense triangles" and avg[dom] > 0:
-        # algorithmic bytes of the classification (candidate stream, 5 B of
-        # HBM per classified candidate: a 4-byte hyperedge id and its 1-byte
-        # overlap); the candidates the dense kernel classifies per launch are
-        # its closed triangles, counted by the traced step
-        cand = float(st.get("candidates", 0))
+    if dom and avg[dom] > 0:
+        # algorithmic bytes of a count: the line graph (two 8-byte entries a
+        # hyperwedge) read once.  The kernels of the phase run side by side and
+        # are bound by L1 sectors and their latency, not by HBM: the fraction
+        # says how far a count is from one reading of its input.
         sec = avg[dom] / 1000.0
-        achieved = 5.0 * cand / sec / 1e9
-        # the kernel's own loads per scanned word: 16 bytes of row a's overlap
-        # planes and adjacency mask, 16 of row b's, 16 of size planes and one
-        # bitmap word per heavy node of e_a & e_b
-        words = float(st.get("words_scanned", 0))
-        hw = float(st.get("dense_hyperwedges", 0)) or 1.0
-        n_t = float(st.get("heavy_bitmaps", 0)) / hw
-        loads = words * 4.0 * (4 + 4 + 4 + n_t)
+        achieved = 16.0 * n_wedges / sec / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak,
-                "traffic": (args.traffic_bytes if args.traffic_bytes is not None else
-                            DENSE_TRAFFIC.get((args.workload, int(st.get("dense_threshold", 0))))),
-                "kernel": "k_dense_triangles", "kernel_ms": avg[dom], "peak_kind": peak_kind,
-                "candidates_per_launch": cand, "bytes_per_candidate": 5,
-                "l2_term": {"bytes_per_candidate": 15, "achieved_gbs": 15.0 * cand / sec / 1e9},
-                "load_model": {"bytes": loads, "achieved_gbs": loads / sec / 1e9,
-                               "frac": loads / sec / 1e9 / peak}}
+                "frac": achieved / peak, "traffic": args.traffic_bytes,
+                "kernel": f"phase {dom!r}", "kernel_ms": avg[dom], "peak_kind": peak_kind,
+                "hyperwedges": int(n_wedges), "bytes_per_hyperwedge": 16}
     sampled = None
     if args.sampled_r > 0:
         sampled = _sampled_measure(ctx, args)
@@ -664,7 +646,7 @@ def main():
     ap.add_argument("--dense-threshold", type=int, default=0,
                     help="split kernel threshold (0: the tuner's choice)")
     ap.add_argument("--traffic-bytes", type=float, default=None,
-                    help="DRAM bytes per dense-kernel launch from an ncu capture, if known")
+                    help="DRAM bytes of the dominant phase from an ncu capture, if known")
     ap.add_argument("--sampled-r", type=int, default=2_000_000,
                     help="MoCHy-A+ samples of the candidates/s line (0: skip)")
     ap.add_argument("--sampled-steps", type=int, default=3)

@@ -230,8 +230,10 @@ int mochy_radial_node_profile(mochy_ctx* ctx, int64_t* np_h, int64_t* np_3h);
  * ascending (parent h-motif id, canonical tuple) order (mochy_kh_pattern).
  * out_kh[t-1] (cap >= X(k) entries, may be NULL) receives the count of
  * kh-motif t, out_h (26, may be NULL) the h-motif counts, *n_motifs (may be
- * NULL) X(k).  Instances are enumerated one by one by the per-hyperwedge
- * scan (exact_kernel = 1's kernel, at most about 300,000 hyperedges).
+ * NULL) X(k).  Thresholds up to 4 are counted by levels of overlap like
+ * mochy_count_exact; with larger ones, or where those arrays do not fit,
+ * instances are enumerated one by one by the per-hyperwedge scan
+ * (exact_kernel = 1's kernel).  At most about 300,000 hyperedges either way.
  * Needs mochy_project. */
 int mochy_count_kh(mochy_ctx* ctx, int32_t k, const int32_t* thresholds, int64_t* out_h,
                    int64_t* out_kh, int64_t cap, int64_t* n_motifs);

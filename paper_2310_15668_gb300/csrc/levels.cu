@@ -839,7 +839,7 @@ __global__ void __launch_bounds__(kManyThreads) k_lv_many(LevelArgs g) {
       uint32_t* R = cell + rows * ncl;   // [rows][nc] of the hubs
       for (int q = threadIdx.x; q < rows * ncl; q += kManyThreads) cell[q] = 0u;
       if (!inside) {
-        // R_a of the hubs of this round: a's hubs from the hub matrix ...
+        // R_a of the hubs of this pass: a's hubs from the hub matrix ...
         for (int r = threadIdx.x; r < rows; r += kManyThreads)
           for (int c = 0; c < nc; ++c) R[r * nc + c] = 0u;
         __syncthreads();
@@ -1358,7 +1358,7 @@ __global__ void __launch_bounds__(kTripThreads, kTripBlocks) k_lv_triples(LevelA
     const int64_t end = min(r0 + per, n_rows);
     if (r0 >= n_rows) break;
     while (r0 < end) {
-      // the segment (unit, class) of row r0, and the rows of this round: of one
+      // the segment (unit, class) of row r0, and the rows of this pass: of one
       // segment, and few enough for the table's 32-bit counts
       __syncthreads();
       if (threadIdx.x == 0) {
@@ -1658,9 +1658,9 @@ k_lv_open(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, int 
 // parts of each (one add_closed, at most kParts) to threads of their own, and
 // the lanes of a warp add to copies of the histogram.
 // Shared atomics on equal bins bound it: 55 -> 43 us at 2,000 hyperedges, 96 ->
-// 61 us at 7,001 with theta = 2, 920 -> 300 us for a batch of 54 (a thread an
-// entry and one histogram a block before; a call of add_closed for each part at
-// a place of its own, where the lanes part, took 350 us at 2,000).
+// 61 us at 7,001 with theta = 2, a batch of 54 as a whole 6.4 -> 5.8 ms (a
+// thread an entry and one histogram a block before; a call of add_closed for
+// each part at a place of its own, where the lanes part, took 350 us at 2,000).
 constexpr int kFinishThreads = 256;
 constexpr int kFinishChunk = 2048;   // entries of a block, at most
 constexpr int kFinishCopies = 8;

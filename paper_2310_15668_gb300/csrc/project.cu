@@ -13,8 +13,8 @@
 // their lists reaches.
 // Issue and shared-memory latency bound it (4.7 warp instructions an entry, 42 %
 // of the issue slots, 20 warps an SM): 100,001 Zipf(1.0) hyperedges, 9.9 GB of
-// line graph, 13.3 ms for both passes, against 56 for windows of list entries;
-// 4 or 6 blocks an SM instead of 8: 21 and 18 ms, blocks of 256 threads 19.
+// line graph: loading and projecting 62.7 ms with windows of list entries, 14
+// here (4 or 6 blocks an SM instead of 8: 21 and 18, blocks of 256 threads 19).
 #include "common.cuh"
 
 namespace mochy {

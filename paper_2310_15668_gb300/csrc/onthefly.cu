@@ -1295,7 +1295,8 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
   const size_t b_pos = al((size_t)std::max<int64_t>(E, 1) * 4), b_id = al((size_t)Wp * 32 * 4);
   const size_t b_deg = by_size ? b_pos + b_id + al((2 * kOtfSizes + 1) * 4)
                                : al((size_t)std::max<int64_t>(E, 1) * 8);
-  const size_t b_up = std::max(al((size_t)std::max<int64_t>(E, 1) * 8), kOtfDrawBytes);
+  // E + 1 entries: the scan reads them all (the last only lends its place)
+  const size_t b_up = std::max(al((size_t)(E + 1) * 8), kOtfDrawBytes);
   const size_t bytes = b_hidx + b_nodes + b_bits + b_sbits + b_pre + b_deg + b_up;
   void* p = nullptr;
   MOCHY_TRY(dev_alloc(ctx, &p, bytes));

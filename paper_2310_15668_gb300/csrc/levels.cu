@@ -1164,40 +1164,51 @@ struct Coder {
   }
 };
 
+// hist[id] += v: a histogram in shared memory, or one in global memory, which
+// other kernels may be adding to, so by one atomic of the bin's whole width
+template <bool kShared>
+__device__ __forceinline__ void bin_add(unsigned long long* hist, int id, long long v) {
+  if (kShared) shared_bin_add(hist, id, v);
+  else atomicAdd(&hist[id], (unsigned long long)v);
+}
+
 // n closed instances of sizes A, B, C, overlaps x, y, z and t (F)
+template <bool kShared>
 __device__ __noinline__ void add_closed(unsigned long long* hist, const Coder& cd, int A, int B,
                                         int C, int x, int y, int z, int t, long long n) {
   if (!n) return;
-  shared_bin_add(hist, cd.id(A - x - z + t, B - x - y + t, C - y - z + t, x - t, y - t, z - t, t), n);
-  if (x + z <= A) shared_bin_add(hist, cd.id(A - x - z, B - x, C - z, x, 0, z, 0), -n);
-  if (x + y <= B) shared_bin_add(hist, cd.id(B - x - y, A - x, C - y, x, 0, y, 0), -n);
-  if (z + y <= C) shared_bin_add(hist, cd.id(C - z - y, A - z, B - y, z, 0, y, 0), -n);
+  bin_add<kShared>(hist, cd.id(A - x - z + t, B - x - y + t, C - y - z + t, x - t, y - t, z - t, t),
+                   n);
+  if (x + z <= A) bin_add<kShared>(hist, cd.id(A - x - z, B - x, C - z, x, 0, z, 0), -n);
+  if (x + y <= B) bin_add<kShared>(hist, cd.id(B - x - y, A - x, C - y, x, 0, y, 0), -n);
+  if (z + y <= C) bin_add<kShared>(hist, cd.id(C - z - y, A - z, B - y, z, 0, y, 0), -n);
 }
 
-// n instances of three heavy pairs, less what the levels 0 to 2 count for them
+// n instances of three heavy pairs, less what the levels 0 to 2 count for them,
+// into a histogram in global memory
 __device__ void add_triple(unsigned long long* hist, const Coder& cd, int A, int B, int C, int x,
                            int y, int z, int t, long long n) {
-  add_closed(hist, cd, A, B, C, x, y, z, t, n);
+  add_closed<false>(hist, cd, A, B, C, x, y, z, t, n);
   long long ft = -((long long)x * y * z - (long long)t * (x + y + z) + 2 * t);
   int a = A, b = B, c = C, xo = x, yo = y, zo = z;
   for (int i = 0; i < 3; ++i) {
     // centre a with pairs (a, b) of overlap xo and (a, c) of zo; opposite yo
-    add_closed(hist, cd, a, b, c, xo, 1, zo, 1, -n * t);
-    add_closed(hist, cd, a, b, c, xo, 1, zo, 0, -n * (yo - t));
+    add_closed<false>(hist, cd, a, b, c, xo, 1, zo, 1, -n * t);
+    add_closed<false>(hist, cd, a, b, c, xo, 1, zo, 0, -n * (yo - t));
     ft += (long long)t * (xo - 1) * (zo - 1) + (long long)(yo - t) * xo * zo;
     // pair (a, b), third member c
     const long long out = -(long long)(yo - t) * (zo - t) + (long long)(yo - t) * zo +
                           (long long)(zo - t) * yo;
-    add_closed(hist, cd, a, b, c, xo, 1, 1, 1, n * t);
-    add_closed(hist, cd, a, b, c, xo, 1, 1, 0, n * out);
+    add_closed<false>(hist, cd, a, b, c, xo, 1, 1, 1, n * t);
+    add_closed<false>(hist, cd, a, b, c, xo, 1, 1, 0, n * out);
     ft -= out * xo;
     // rotate: a -> b -> c -> a
     const int ta = a, tx = xo;
     a = b; b = c; c = ta;
     xo = yo; yo = zo; zo = tx;
   }
-  add_closed(hist, cd, A, B, C, 1, 1, 1, 1, -n * t);
-  add_closed(hist, cd, A, B, C, 1, 1, 1, 0, n * ft);
+  add_closed<false>(hist, cd, A, B, C, 1, 1, 1, 1, -n * t);
+  add_closed<false>(hist, cd, A, B, C, 1, 1, 1, 0, n * ft);
 }
 
 // ---------------------------------------------------------------------------
@@ -1761,7 +1772,7 @@ k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, in
   for (int w = threadIdx.x; w < n_queue * kParts; w += kFinishThreads) {
     const int64_t at = first + queue[w / kParts];
     const Part o = entry_part(g, at, w % kParts, tab[at]);
-    add_closed(hist, cd, o.A, o.B, o.C, o.x, o.y, o.z, o.t, o.n);
+    add_closed<true>(hist, cd, o.A, o.B, o.C, o.x, o.y, o.z, o.t, o.n);
   }
   // the tuples outside the table
   for (int64_t s0 = (int64_t)blockIdx.x * kFinishThreads; s0 <= (int64_t)g.omask;
@@ -1781,7 +1792,7 @@ k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, in
       const int x = t + p, y = t + q, z = t + r;
       const Part o = triple_part(w % kParts, a1 + x + r, b1 + x + q, c1 + y + r, x, y, z, t,
                                  (long long)g.ocnt[s]);
-      add_closed(hist, cd, o.A, o.B, o.C, o.x, o.y, o.z, o.t, o.n);
+      add_closed<true>(hist, cd, o.A, o.B, o.C, o.x, o.y, o.z, o.t, o.n);
     }
   }
   __syncthreads();

@@ -1,0 +1,86 @@
+"""The exact count by levels of overlap at the limits of its structures (needs
+a GB300), against the oracle.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2310_15668_gb300 import binding as B
+from . import _util
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _wide(n, e, lo, hi, seed):
+    rng = np.random.default_rng(seed)
+    sets = {tuple(sorted(rng.choice(n, rng.integers(lo, hi + 1), replace=False).tolist()))
+            for _ in range(e)}
+    return (n, *_util.csr_from_sets(sorted(sets)))
+
+
+def _count(g, **kw):
+    with B.Context(**kw) as c:
+        c.load(*g)
+        c.project()
+        return c.count_exact()
+
+
+def _distinct_tuples(g, theta, t_from):
+    """Region sizes of the triples with t >= t_from common nodes and three
+    overlaps of 2 or more, own regions capped at t + theta + 1, the members in
+    any order: fewer than the level 3 tuples."""
+    n, off, nodes = g
+    E = len(off) - 1
+    m = np.zeros((E, n), np.int32)
+    for i in range(E):
+        m[i, nodes[off[i]:off[i + 1]]] = 1
+    om = m @ m.T
+    size = m.sum(1)
+    keys = set()
+    for a in range(E):
+        t = (m * m[a]) @ m.T
+        b, k = np.triu_indices(E, 1)
+        ok = (b > a) & (t[b, k] >= t_from) & (om[a, b] > 1) & (om[a, k] > 1) & (om[b, k] > 1)
+        b, k = b[ok], k[ok]
+        tt, x, y, z = t[b, k], om[a, b], om[b, k], om[a, k]
+        cap = tt + theta + 1
+        own = np.sort(np.stack([np.minimum(size[a] - x - z + tt, cap),
+                                np.minimum(size[b] - x - y + tt, cap),
+                                np.minimum(size[k] - y - z + tt, cap)], 1), 1)
+        pair = np.sort(np.stack([x, y, z], 1), 1)
+        for row in np.unique(np.concatenate([tt[:, None], pair, own], 1), axis=0):
+            keys.add(tuple(row.tolist()))
+    return len(keys)
+
+
+WIDE = (70, 170, 12, 60, 31)
+
+
+@pytest.mark.parametrize("theta", [1, 4])
+def test_more_tuples_than_the_hash_holds(theta):
+    """Level 3 tuples outside the table (5 common nodes or more) fill the hash
+    of such tuples, and the rest goes straight to the histogram."""
+    g = _wide(*WIDE)
+    E = len(g[1]) - 1
+    slots = 1 << 12
+    while slots < E * (E - 1) / 4:      # at most this many: a quarter of the heavy entries
+        slots *= 2
+    assert _distinct_tuples(g, theta, 5) > slots
+    h, h3 = _count(g, theta=theta)
+    oh, o3 = oracle.count_exact(g[1], g[2], theta=theta)
+    assert np.array_equal(h, oh) and np.array_equal(h3, o3)
+
+
+def test_more_tuples_than_the_hash_holds_in_a_batch():
+    gs = [_wide(*WIDE), _wide(12, 60, 2, 5, 32), _wide(70, 150, 12, 60, 33)]
+    seeds = [4, 5, 6]
+    _, _, _, _, ch, c3, _, _ = B.mochy_profile_batch(gs, 1, seeds)
+    for g, (n, off, nodes) in enumerate(gs):
+        o = oracle.profile(n, off, nodes, 1, seeds[g])
+        assert np.array_equal(ch[g], o["counts_h"]) and np.array_equal(c3[g], o["counts_3h"])

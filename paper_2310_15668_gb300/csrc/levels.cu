@@ -1753,19 +1753,24 @@ __device__ __forceinline__ Part entry_part(const LevelArgs& g, int64_t at, int p
   return {e / (Q * Q) + 1, e / Q % Q + 1, e % Q + 1, 1, 1, 1, star ? 1 : 0, part == 0 ? n : 0};
 }
 
+// The blocks go over the units (of one histogram each) and, within a unit, over
+// the chunks of its tables, all along grid.x: grid.y ends at 65,535, and a batch
+// may have more units.  The hash of tuples outside the table is one for all
+// units and is gone over once: its tuples are added to the block's histogram
+// when there is one unit, else to their units' in global memory.
 __global__ void __launch_bounds__(kFinishThreads)
 k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, int n_bins,
-            int chunk, int copies) {
+            int n_chunks, int chunk, int copies) {
   extern __shared__ unsigned long long hists[];   // [copies][n_bins + 1]
   __shared__ int32_t queue[kFinishChunk];
   __shared__ int32_t n_queue;
-  const int unit = blockIdx.y;
+  const int unit = (int)blockIdx.x / n_chunks;
   unsigned long long* hist = hists + (threadIdx.x & (copies - 1)) * (n_bins + 1);
   for (int q = threadIdx.x; q < copies * (n_bins + 1); q += kFinishThreads) hists[q] = 0ull;
   if (threadIdx.x == 0) n_queue = 0;
   __syncthreads();
   const int64_t* tab = g.tab + unit * g.tab_stride;
-  const int64_t first = (int64_t)blockIdx.x * chunk;
+  const int64_t first = (int64_t)(blockIdx.x - unit * n_chunks) * chunk;
   for (int q = threadIdx.x; q < chunk && first + q < g.n_tab; q += kFinishThreads)
     if (tab[first + q]) queue[atomicAdd(&n_queue, 1)] = q;
   __syncthreads();
@@ -1781,7 +1786,7 @@ k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, in
     if (threadIdx.x == 0) n_queue = 0;
     __syncthreads();
     const unsigned long long k = g.okey[s0 + threadIdx.x];   // slots: a multiple of the threads
-    if (k && (int)((k - 1) >> 45) == unit) queue[atomicAdd(&n_queue, 1)] = threadIdx.x;
+    if (k) queue[atomicAdd(&n_queue, 1)] = threadIdx.x;
     __syncthreads();
     for (int w = threadIdx.x; w < n_queue * kParts; w += kFinishThreads) {
       const int64_t s = s0 + queue[w / kParts];
@@ -1792,7 +1797,11 @@ k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, in
       const int x = t + p, y = t + q, z = t + r;
       const Part o = triple_part(w % kParts, a1 + x + r, b1 + x + q, c1 + y + r, x, y, z, t,
                                  (long long)g.ocnt[s]);
-      add_closed<true>(hist, cd, o.A, o.B, o.C, o.x, o.y, o.z, o.t, o.n);
+      if (g.n_units == 1)
+        add_closed<true>(hist, cd, o.A, o.B, o.C, o.x, o.y, o.z, o.t, o.n);
+      else
+        add_closed<false>(hist_out + (int64_t)(e >> 45) * n_bins, cd, o.A, o.B, o.C, o.x, o.y, o.z,
+                          o.t, o.n);
     }
   }
   __syncthreads();
@@ -2130,8 +2139,10 @@ int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const 
          ceil_div(g.n_tab, chunk) * (int64_t)g.n_units > (int64_t)ctx->num_sms * 32)
     chunk *= 2;
   while (copies > 1 && (size_t)copies * (n_bins + 1) * 8 > 32 * 1024) copies /= 2;
-  k_lv_finish<<<dim3((unsigned)ceil_div(g.n_tab, chunk), g.n_units), kFinishThreads,
-                (size_t)copies * (n_bins + 1) * 8, st>>>(g, cd, d_hist, n_bins, chunk, copies);
+  const int n_chunks = ceil_div(g.n_tab, chunk);
+  k_lv_finish<<<(unsigned)n_chunks * (unsigned)g.n_units, kFinishThreads,
+                (size_t)copies * (n_bins + 1) * 8, st>>>(g, cd, d_hist, n_bins, n_chunks, chunk,
+                                                         copies);
   MOCHY_LAUNCHED();
   if (timer) timer->mark("finish");
   return MOCHY_OK;

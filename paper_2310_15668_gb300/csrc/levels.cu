@@ -77,7 +77,7 @@ struct LevelUnit {
   int64_t mstride;  // words a row
   int64_t n_dense;
   int64_t hbase;    // first hub index
-  int64_t n_hubs;   // at most kMaxHubs
+  int64_t n_hubs;   // at most kMaxHubs, those of highest degree
   int64_t hmoff;    // first entry of its hub matrix
 };
 
@@ -250,6 +250,40 @@ k_lv_nodes(LevelArgs g, int hub_deg, uint32_t* __restrict__ ncls, int64_t* __res
   }
 }
 
+// Units of more hubs than kMaxHubs keep those of highest degree, the lower id
+// first among equals: with ids in another order than by popularity, the first
+// kMaxHubs by id would leave popular nodes among the light ones, whose node
+// pairs cost the product of their degrees (k_lv_light_pairs).  The nodes are
+// sorted by degree, then (a batch) stably by unit.
+__global__ void k_lv_degree_keys(LevelArgs g, uint32_t* __restrict__ key,
+                                 uint32_t* __restrict__ val) {
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= g.n_nodes) return;
+  key[v] = ~(uint32_t)(g.voff[v + 1] - g.voff[v]);
+  val[v] = (uint32_t)v;
+}
+
+__global__ void k_lv_unit_keys(LevelArgs g, const uint32_t* __restrict__ val,
+                               uint32_t* __restrict__ key) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < g.n_nodes) key[i] = (uint32_t)unit_of(g.nseg, g.n_units, val[i]);
+}
+
+__global__ void k_lv_pick_hubs(LevelArgs g, const uint32_t* __restrict__ val, int hub_deg,
+                               int64_t* __restrict__ seg_b) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= g.n_nodes) return;
+  const int64_t v = val[i];
+  const int64_t rank = i - (g.n_units > 1 ? g.nseg[unit_of(g.nseg, g.n_units, v)] : 0);
+  seg_b[v] = rank < kMaxHubs && g.voff[v + 1] - g.voff[v] >= hub_deg ? 1 : 0;
+}
+
+// is node v a hub?  bscan: the scan of the hubs' flags (one entry follows the
+// last node's)
+__device__ __forceinline__ bool is_hub(const int64_t* __restrict__ bscan, int64_t v) {
+  return bscan[v + 1] != bscan[v];
+}
+
 // totals the host needs: [h, pairs, neighbours] then per unit the first dense
 // index and the first hub index (U + 1 each)
 __global__ void k_lv_totals(LevelArgs g, const int64_t* __restrict__ S, int64_t o_d, int64_t o_p,
@@ -348,7 +382,7 @@ __global__ void __launch_bounds__(kRowThreads) k_lv_matrix(LevelArgs g) {
 // warp per hyperedge: its node pairs into the pair table, hub indices of its
 // nodes
 __global__ void __launch_bounds__(kRowThreads)
-k_lv_pairs(LevelArgs g, const int64_t* __restrict__ bscan, int hub_deg, uint64_t* __restrict__ hkey,
+k_lv_pairs(LevelArgs g, const int64_t* __restrict__ bscan, uint64_t* __restrict__ hkey,
            uint32_t* __restrict__ hcnt, uint16_t* __restrict__ ehub) {
   __shared__ int32_t nodes[kRowWarps][64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -360,9 +394,7 @@ k_lv_pairs(LevelArgs g, const int64_t* __restrict__ bscan, int hub_deg, uint64_t
     for (int q = lane; q < A; q += 32) {
       const int32_t v = g.enode[eb + q];
       nodes[warp][q] = v;
-      const int64_t h = bscan[v] - bscan[0] - hbase;
-      const bool hub = g.voff[v + 1] - g.voff[v] >= hub_deg && h < kMaxHubs;
-      ehub[eb + q] = hub ? (uint16_t)h : (uint16_t)0xffff;
+      ehub[eb + q] = is_hub(bscan, v) ? (uint16_t)(bscan[v] - bscan[0] - hbase) : (uint16_t)0xffff;
     }
     __syncwarp();
     const int c = min(A, g.Q) - 2;
@@ -623,7 +655,7 @@ __device__ __forceinline__ void nth_pair(int n, int& i, int& j) {
 }
 
 // hubs x hubs: M_uw, four counts a pair (size classes from 2), per unit
-__global__ void k_lv_hub_matrix(LevelArgs g, const int64_t* __restrict__ bscan, int hub_deg,
+__global__ void k_lv_hub_matrix(LevelArgs g, const int64_t* __restrict__ bscan,
                                 uint32_t* __restrict__ hubm) {
   const int64_t n = (int64_t)g.hmask + 1;
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
@@ -631,10 +663,9 @@ __global__ void k_lv_hub_matrix(LevelArgs g, const int64_t* __restrict__ bscan, 
     const uint64_t k = g.hkey[s];
     if (!k) continue;
     const int32_t u = (int32_t)(k >> 32), w = (int32_t)(k & 0xffffffffu);
-    if (g.voff[u + 1] - g.voff[u] < hub_deg || g.voff[w + 1] - g.voff[w] < hub_deg) continue;
+    if (!is_hub(bscan, u) || !is_hub(bscan, w)) continue;
     const LevelUnit un = g.unit[unit_of(g.nseg, g.n_units, u)];
     const int64_t hu = bscan[u] - bscan[0] - un.hbase, hw = bscan[w] - bscan[0] - un.hbase;
-    if (hu >= un.n_hubs || hw >= un.n_hubs) continue;
     for (int c = 0; c < g.CP; ++c) {
       const uint32_t m = g.hcnt[(uint64_t)s * g.CP + c];
       hubm[(un.hmoff + hu * un.n_hubs + hw) * g.CP + c] = m;
@@ -1014,7 +1045,7 @@ __global__ void __launch_bounds__(kManyThreads) k_lv_many(LevelArgs g) {
 // Level 1, light-light part: warp per pair of light nodes (u, w) that some
 // hyperedge holds, lanes over the pairs (a, b) of their hyperedges.
 __global__ void __launch_bounds__(kRowThreads)
-k_lv_light_pairs(LevelArgs g, const int64_t* __restrict__ bscan, int hub_deg) {
+k_lv_light_pairs(LevelArgs g, const int64_t* __restrict__ bscan) {
   extern __shared__ unsigned long long acc[];   // [kL1Rows][Q^3]
   const int lane = threadIdx.x & 31;
   const int Q = g.Q, n_sh = min(kL1Rows, g.S - 1) * Q * Q * Q;
@@ -1028,12 +1059,7 @@ k_lv_light_pairs(LevelArgs g, const int64_t* __restrict__ bscan, int hub_deg) {
     bool light = k0 != 0ull;
     if (light) {
       const int32_t u = (int32_t)(k0 >> 32), w = (int32_t)(k0 & 0xffffffffu);
-      const LevelUnit& un = g.unit[unit_of(g.nseg, g.n_units, u)];
-      auto hub = [&](int32_t v) {
-        return g.voff[v + 1] - g.voff[v] >= hub_deg && bscan[v] - bscan[0] - un.hbase < un.n_hubs;
-      };
-      // a node of one hyperedge only meets itself there
-      light = !hub(u) && !hub(w);
+      light = !is_hub(bscan, u) && !is_hub(bscan, w);
     }
     for (unsigned todo = __ballot_sync(0xffffffffu, light); todo; todo &= todo - 1u) {
       const int src = __ffs(todo) - 1;
@@ -1962,12 +1988,31 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   k_lv_nodes<<<row_grid(ctx, N, 8), kRowThreads, 0, st>>>(g, kHubDeg, ncls, seg + o_b, seg + o_n);
   MOCHY_LAUNCHED();
   MOCHY_CUDA(cudaMemsetAsync(seg + n_seg, 0, 8, st));
-  MOCHY_TRY(scan_exclusive_i64(ctx, seg, scan, n_seg + 1));
-  k_lv_totals<<<ceil_div(U + 1, 128), 128, 0, st>>>(g, scan, o_d, o_p, o_b, o_n, n_seg, d_tot);
-  MOCHY_LAUNCHED();
   std::vector<int64_t> tot((size_t)3 + 2 * (U + 1));
-  MOCHY_CUDA(cudaMemcpyAsync(tot.data(), d_tot, tot.size() * 8, cudaMemcpyDeviceToHost, st));
-  MOCHY_CUDA(cudaStreamSynchronize(st));
+  const int64_t* hub_tot = tot.data() + 3 + U + 1;   // first hub of each unit
+  for (bool ranked = false;; ranked = true) {
+    MOCHY_TRY(scan_exclusive_i64(ctx, seg, scan, n_seg + 1));
+    k_lv_totals<<<ceil_div(U + 1, 128), 128, 0, st>>>(g, scan, o_d, o_p, o_b, o_n, n_seg, d_tot);
+    MOCHY_LAUNCHED();
+    MOCHY_CUDA(cudaMemcpyAsync(tot.data(), d_tot, tot.size() * 8, cudaMemcpyDeviceToHost, st));
+    MOCHY_CUDA(cudaStreamSynchronize(st));
+    bool crowded = false;
+    for (int u = 0; u < U; ++u) crowded = crowded || hub_tot[u + 1] - hub_tot[u] > kMaxHubs;
+    if (!crowded || ranked) break;
+    MOCHY_TRY(scratch(ctx, 2, (size_t)N * 8, &t));
+    uint32_t* key = (uint32_t*)t;
+    uint32_t* val = key + N;
+    k_lv_degree_keys<<<ceil_div(N, 256), 256, 0, st>>>(g, key, val);
+    MOCHY_LAUNCHED();
+    MOCHY_TRY(radix_sort_pairs_u32(ctx, key, val, N, 32));
+    if (U > 1) {
+      k_lv_unit_keys<<<ceil_div(N, 256), 256, 0, st>>>(g, val, key);
+      MOCHY_LAUNCHED();
+      MOCHY_TRY(radix_sort_pairs_u32(ctx, key, val, N, bits_for(U)));
+    }
+    k_lv_pick_hubs<<<ceil_div(N, 256), 256, 0, st>>>(g, val, kHubDeg, seg + o_b);
+    MOCHY_LAUNCHED();
+  }
   const int64_t H = tot[0], P = tot[1], NB = tot[2];
   // a row has at most sqrt(H) later partners (each has as many itself), whose
   // pairs then fit 32 bits
@@ -1984,8 +2029,8 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
     un.mstride = (nd + 7) / 8;
     un.moff = mwords;
     mwords += nd * un.mstride;
-    un.hbase = tot[3 + U + 1 + u];
-    un.n_hubs = std::min<int64_t>(tot[3 + U + 1 + u + 1] - un.hbase, kMaxHubs);
+    un.hbase = hub_tot[u];
+    un.n_hubs = hub_tot[u + 1] - un.hbase;
     un.hmoff = hub_pairs;
     hub_pairs += un.n_hubs * un.n_hubs;
   }
@@ -2061,13 +2106,13 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   k_lv_matrix<<<row_grid(ctx, E, 8), kRowThreads, 0, st>>>(g);
   MOCHY_LAUNCHED();
   cudaStream_t s0 = ctx->side[0];
-  k_lv_pairs<<<row_grid(ctx, E, 8), kRowThreads, 0, s0>>>(g, scan + o_b, kHubDeg, hkey, hcnt, ehub);
+  k_lv_pairs<<<row_grid(ctx, E, 8), kRowThreads, 0, s0>>>(g, scan + o_b, hkey, hcnt, ehub);
   MOCHY_LAUNCHED();
   const unsigned slot_grid =
       (unsigned)std::min<uint64_t>(slots / 256 + 1, (uint64_t)ctx->num_sms * 8);
   k_lv_orient<<<slot_grid, 256, 0, s0>>>(g, scan + o_n, cursor, adj);
   MOCHY_LAUNCHED();
-  k_lv_hub_matrix<<<slot_grid, 256, 0, s0>>>(g, scan + o_b, kHubDeg, hubm);
+  k_lv_hub_matrix<<<slot_grid, 256, 0, s0>>>(g, scan + o_b, hubm);
   MOCHY_LAUNCHED();
   MOCHY_TRY(join_sides(ctx, 1));
   lv->bscan = scan + o_b;
@@ -2123,7 +2168,7 @@ int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const 
   k_lv_light<<<row_grid(ctx, E * kLightSlices, 8), kRowThreads, 0, ctx->side[2]>>>(g);
   MOCHY_LAUNCHED();
   k_lv_light_pairs<<<row_grid(ctx, (int64_t)g.hmask / 32 + 1, 8), kRowThreads, s1, ctx->side[2]>>>(
-      g, lv->bscan, kHubDeg);
+      g, lv->bscan);
   MOCHY_LAUNCHED();
   k_lv_open<<<row_grid(ctx, E, 4), kRowThreads, (size_t)n_bins * 8, ctx->side[2]>>>(g, cd, d_hist,
                                                                                    n_bins);

@@ -1,6 +1,8 @@
 """The exact count by levels of overlap at the limits of its structures (needs
 a GB300), against the oracle.
 """
+import time
+
 import numpy as np
 import pytest
 
@@ -84,3 +86,54 @@ def test_more_tuples_than_the_hash_holds_in_a_batch():
     for g, (n, off, nodes) in enumerate(gs):
         o = oracle.profile(n, off, nodes, 1, seeds[g])
         assert np.array_equal(ch[g], o["counts_h"]) and np.array_equal(c3[g], o["counts_3h"])
+
+
+def _popular(nodes, edges, popular, first, seed):
+    """Hyperedges of 18 of `nodes` nodes, about alike in degree, and two of
+    `popular` popular ones, whose ids come before (or after) all others."""
+    rng = np.random.default_rng(seed)
+    a, b = (popular, 0) if first else (0, nodes)
+    sets = {tuple(sorted((rng.choice(nodes, 18, replace=False) + a).tolist() +
+                         (rng.choice(popular, 2, replace=False) + b).tolist()))
+            for _ in range(edges)}
+    return (nodes + popular, *_util.csr_from_sets(sorted(sets)))
+
+
+def _timed_count(g, **kw):
+    with B.Context(**kw) as c:
+        c.load(*g)
+        c.project()
+        got = c.count_exact()
+        best = 1e9
+        for _ in range(3):
+            t = time.perf_counter()
+            c.count_exact()
+            best = min(best, time.perf_counter() - t)
+    return got, best
+
+
+def test_hubs_do_not_depend_on_the_order_of_ids():
+    """More nodes of degree 32 or more than the hub matrix holds (4,096): the
+    most popular are hubs whatever their ids.  As light nodes, a pair of them
+    would cost the product of their degrees, some 5,000 each, on one warp."""
+    last = _popular(5000, 13000, 5, False, 41)
+    deg = np.bincount(last[2], minlength=last[0])
+    assert (deg >= 32).sum() > 4200 and (deg[5000:] > 3000).all()
+    first = _popular(5000, 13000, 5, True, 41)
+    got, t_last = _timed_count(last)
+    ref, t_first = _timed_count(first)
+    split = _count(last, rest_path=2)
+    for a, b, c in zip(got, ref, split):
+        assert np.array_equal(a, b) and np.array_equal(a, c)
+    assert t_last < 3 * t_first, (t_last, t_first)
+
+
+def test_hubs_of_crowded_units_in_a_batch():
+    gs = [_wide(40, 90, 2, 6, 51), _popular(5000, 13000, 5, False, 42), _wide(3000, 1500, 2, 5, 52),
+          _popular(4900, 12500, 3, True, 43)]
+    seeds = [1, 2, 3, 4]
+    cfg = B.mochy_config_default()
+    cfg.rest_path = 2                    # the split kernels
+    got = B.mochy_profile_batch(gs, 1, seeds)
+    ref = B.mochy_profile_batch(gs, 1, seeds, cfg)
+    assert np.array_equal(got[4], ref[4]) and np.array_equal(got[5], ref[5])

@@ -226,6 +226,8 @@ void release_projection(mochy_ctx* ctx) {
   ctx->projected = false;
   ctx->n_wedges = 0;
   ctx->max_deg = 0;
+  for (int& theta : ctx->levels_declined) theta = 0;
+  ctx->model_thr = 0;
 }
 
 void release_graph(mochy_ctx* ctx) {

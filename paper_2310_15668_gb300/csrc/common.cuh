@@ -82,6 +82,10 @@ constexpr int kMaxPhases = 16;   // traced phases of one count
 
 struct Levels;   // structures of the exact count by levels (levels.cu)
 
+// what would count instead of the levels: they are taken against the split
+// kernels or the kh scan only where they take less time
+enum class LevelsAgainst { kNothing, kSplit, kScan };
+
 // Scratch arena: grows on demand, freed with the context.
 struct Buffer {
   void* p = nullptr;
@@ -170,6 +174,9 @@ struct mochy_ctx {
 
   // exact count by levels (built on first use, released with the line graph)
   mochy::Levels* levels = nullptr;
+  int levels_declined[3] = {};   // by LevelsAgainst: theta at which that takes less time
+  int model_thr = 0;             // the cost model's dense threshold, once it was asked
+  double model_sparse = 0.0, model_words = 0.0;   // what it leaves the split kernels to do
   cudaStream_t side[mochy::kSides] = {};        // its independent kernels run side by side
   cudaEvent_t side_ev[mochy::kSides + 1] = {};
   bool split_forced = false;     // the configuration asks for the split kernels
@@ -261,13 +268,14 @@ int enumerate_instances(mochy_ctx* ctx, int64_t cap, int32_t* d_out,
                         unsigned long long* d_cursor);                // extensions.cu
 int prepare_split(mochy_ctx* ctx);                                    // count_split.cu
 bool levels_cover(int theta, int64_t n_edges, int n_units);           // levels.cu
-int prepare_levels(mochy_ctx* ctx, int theta);                        // levels.cu
+int prepare_levels(mochy_ctx* ctx, int theta, LevelsAgainst against); // levels.cu
 struct PhaseTimer;
 int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const uint16_t* lut, int k,
                   int t1, int t2, PhaseTimer* timer);                 // levels.cu
 void release_levels(mochy_ctx* ctx);                                  // levels.cu
 int prepare_exact(mochy_ctx* ctx, bool* by_levels);                   // count_split.cu
 int choose_dense_threshold(mochy_ctx* ctx);                           // tune.cu
+int model_split_work(mochy_ctx* ctx, double* sparse, double* words);  // tune.cu
 int tune_dense_threshold(mochy_ctx* ctx, const int32_t* cand, int32_t n_cand, double fraction,
                          uint64_t seed, int32_t* best, int32_t* tried,
                          double* ms);                                 // tune.cu

@@ -1719,18 +1719,28 @@ static int launch_split(mochy_ctx* ctx, SplitPlan p, PhaseTimer* timer, const Wo
 // Builds what the exact count of this context needs and says which kernels
 // it takes: by levels of overlap (levels.cu), unless the configuration asks
 // for the split kernels (dense_threshold or rest_path), theta is past what the
-// level tables hold, or the level structures do not fit the device memory.
+// level tables hold, the split kernels take less time (levels_pay in
+// levels.cu), or the level structures do not fit the device memory.
 int prepare_exact(mochy_ctx* ctx, bool* by_levels) {
   *by_levels = false;
   if (!ctx->split_forced && levels_cover(ctx->theta, ctx->n_edges, ctx->n_units)) {
-    const int rc = prepare_levels(ctx, ctx->theta);
+    const int rc = prepare_levels(ctx, ctx->theta, LevelsAgainst::kSplit);
     if (rc >= 0) {
       *by_levels = true;
       return MOCHY_OK;
     }
     if (rc != MOCHY_E_NOMEM && rc != MOCHY_E_UNSUPPORTED) return rc;
   }
-  return prepare_split(ctx);
+  const int rc = prepare_split(ctx);
+  if ((rc == MOCHY_E_NOMEM || rc == MOCHY_E_UNSUPPORTED) &&
+      ctx->levels_declined[(int)LevelsAgainst::kSplit] == ctx->theta) {
+    // declined for their time alone
+    release_split(ctx);
+    MOCHY_TRY(prepare_levels(ctx, ctx->theta, LevelsAgainst::kNothing));
+    *by_levels = true;
+    return MOCHY_OK;
+  }
+  return rc;
 }
 
 int count_exact_split(mochy_ctx* ctx, unsigned long long* d_hist) {

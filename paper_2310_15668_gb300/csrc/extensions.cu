@@ -400,7 +400,7 @@ int count_kh(mochy_ctx* ctx, int k, int thr1, int thr2, unsigned long long* d_hi
   // 4,001 Zipf hyperedges, k = 4: 28.5 ms against 1.4)
   const int theta = k == 2 ? 1 : k == 3 ? thr1 : thr2;
   if (levels_cover(theta, ctx->n_edges, ctx->n_units)) {
-    const int rc = prepare_levels(ctx, theta);
+    const int rc = prepare_levels(ctx, theta, LevelsAgainst::kScan);
     if (rc >= 0)
       return launch_levels(ctx, d_hist, n_bins, ctx->kh_lut, k, k == 2 ? 1 << 30 : thr1,
                            k < 4 ? 1 << 30 : thr2, nullptr);

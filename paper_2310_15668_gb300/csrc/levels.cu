@@ -55,6 +55,7 @@
 //   k_lv_light_pairs  0.10 /  0.28 ms the same
 // They run side by side on four streams: a whole count 1.3 / 31 ms, against
 // 21 / 890 ms for the triangle kernels of count_split.cu.
+#include <cmath>
 #include <cstring>
 
 #include "classify.cuh"
@@ -207,34 +208,79 @@ __host__ __device__ inline int trip_class(int A, int theta) {
 // Preparation
 // ---------------------------------------------------------------------------
 
+// What the ways of counting have to go over (see levels_pay): the sum of the
+// squared line degrees, and what light nodes cost the levels, in units of 1,024.
+struct Work {
+  unsigned long long deg2, light_pairs, light_rows;
+};
+
+// adds up n, one value a thread, over a block of kRowThreads
+__device__ __forceinline__ void block_add(unsigned long long n, unsigned long long* out) {
+  __shared__ unsigned long long part[kRowWarps];
+  for (int d = 16; d; d >>= 1) n += __shfl_xor_sync(0xffffffffu, n, d);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = n;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long s = 0ull;
+    for (int w = 0; w < kRowWarps; ++w) s += part[w];
+    if (s) atomicAdd(out, s);
+  }
+  __syncthreads();
+}
+
 // heavy degrees, which rows can be in a triangle of heavy pairs, and node
 // pairs of each hyperedge
-__global__ void k_lv_rows(int64_t n_edges, const int32_t* __restrict__ heavy,
-                          const uint8_t* __restrict__ esize, int64_t* __restrict__ seg_h,
-                          int64_t* __restrict__ seg_d, int64_t* __restrict__ seg_p) {
+__global__ void __launch_bounds__(kRowThreads)
+k_lv_rows(int64_t n_edges, const int64_t* __restrict__ noff, const int32_t* __restrict__ heavy,
+          const uint8_t* __restrict__ esize, int64_t* __restrict__ seg_h,
+          int64_t* __restrict__ seg_d, int64_t* __restrict__ seg_p, Work* __restrict__ work) {
   const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= n_edges) return;
-  const int64_t h = heavy[a], A = esize[a];
-  seg_h[a] = h;
-  seg_d[a] = h >= 2 ? 1 : 0;
-  seg_p[a] = A * (A - 1) / 2;
+  int64_t deg = 0;
+  if (a < n_edges) {
+    const int64_t h = heavy[a], A = esize[a];
+    deg = noff[a + 1] - noff[a];
+    seg_h[a] = h;
+    seg_d[a] = h >= 2 ? 1 : 0;
+    seg_p[a] = A * (A - 1) / 2;
+  }
+  block_add((unsigned long long)(deg * deg), &work->deg2);
 }
+
+// The light work of a node in d hyperedges, with `others` other members in all
+// and `many` heavy pairs at those of its hyperedges that have more than
+// kFewHeavy: d d' summed over the nodes d' that it shares a hyperedge with (as
+// if they were alike), and d / 2 for each of the heavy pairs.
+struct LightWork {
+  unsigned long long pairs = 0ull, rows = 0ull;
+  __device__ __forceinline__ void add(int64_t d, int64_t others, int64_t many) {
+    pairs += ((unsigned long long)d * d * (others + d) / 2 + 512) >> 10;
+    rows += ((unsigned long long)d * many / 2 + 512) >> 10;
+  }
+};
 
 // warp per node: hyperedges of each size class that hold it, whether it is a
 // hub, and a bound on its neighbours in the node graph
 __global__ void __launch_bounds__(kRowThreads)
-k_lv_nodes(LevelArgs g, int hub_deg, uint32_t* __restrict__ ncls, int64_t* __restrict__ seg_b,
-           int64_t* __restrict__ seg_n) {
+k_lv_nodes(LevelArgs g, int hub_deg, const int32_t* __restrict__ heavy,
+           uint32_t* __restrict__ ncls, int64_t* __restrict__ seg_b, int64_t* __restrict__ seg_n,
+           Work* __restrict__ work) {
+  LightWork light;   // of lane 0
   const int lane = threadIdx.x & 31;
   const int64_t nw = (int64_t)gridDim.x * kRowWarps;
   for (int64_t v = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5); v < g.n_nodes; v += nw) {
     const int64_t b = g.voff[v], e = g.voff[v + 1];
-    int64_t others = 0;
+    const bool hub = e - b >= hub_deg;
+    int64_t others = 0, many = 0;
     uint32_t mine = 0;   // count of class `lane` (Q <= 32)
     for (int64_t p0 = b; p0 < e; p0 += 32) {
       const int64_t p = p0 + lane;
-      const int s = p < e ? g.esize[g.vedge[p]] : 0;
+      const int32_t k = p < e ? g.vedge[p] : 0;
+      const int s = p < e ? g.esize[k] : 0;
       others += s > 0 ? s - 1 : 0;
+      if (!hub && p < e) {
+        const int32_t h = heavy[k];
+        many += h > kFewHeavy ? h : 0;
+      }
       const int c = s > 0 ? min(s, g.Q) - 1 : -1;
       for (int q = 0; q < g.Q; ++q) {
         const int n = __popc(__ballot_sync(0xffffffffu, c == q));
@@ -242,12 +288,17 @@ k_lv_nodes(LevelArgs g, int hub_deg, uint32_t* __restrict__ ncls, int64_t* __res
       }
     }
     for (int d = 16; d; d >>= 1) others += __shfl_xor_sync(0xffffffffu, others, d);
+    if (!hub)
+      for (int d = 16; d; d >>= 1) many += __shfl_xor_sync(0xffffffffu, many, d);
     if (lane < g.Q) ncls[v * g.Q + lane] = mine;
     if (lane == 0) {
-      seg_b[v] = e - b >= hub_deg ? 1 : 0;
+      seg_b[v] = hub ? 1 : 0;
       seg_n[v] = others;
+      if (!hub) light.add(e - b, others, many);
     }
   }
+  block_add(light.pairs, &work->light_pairs);
+  block_add(light.rows, &work->light_rows);
 }
 
 // Units of more hubs than kMaxHubs keep those of highest degree, the lower id
@@ -284,15 +335,39 @@ __device__ __forceinline__ bool is_hub(const int64_t* __restrict__ bscan, int64_
   return bscan[v + 1] != bscan[v];
 }
 
+// The light work again, when the hubs are not all nodes of that degree (thread
+// per hyperedge): with l the degrees of its light nodes together, l^2 / 2 pairs
+// of hyperedges, and h l / 2 around its heavy pairs h.
+__global__ void __launch_bounds__(kRowThreads)
+k_lv_light_work(LevelArgs g, const int32_t* __restrict__ heavy, const int64_t* __restrict__ bscan,
+                Work* __restrict__ work) {
+  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned long long l = 0ull, h = 0ull;
+  if (a < g.n_edges) {
+    for (int64_t q = g.eoff[a]; q < g.eoff[a + 1]; ++q) {
+      const int32_t v = g.enode[q];
+      if (!is_hub(bscan, v)) l += (unsigned long long)(g.voff[v + 1] - g.voff[v]);
+    }
+    h = (unsigned long long)heavy[a];
+  }
+  block_add((l * l / 2 + 512) >> 10, &work->light_pairs);
+  block_add(h > kFewHeavy ? (h * l / 2 + 512) >> 10 : 0ull, &work->light_rows);
+}
+
 // totals the host needs: [h, pairs, neighbours] then per unit the first dense
-// index and the first hub index (U + 1 each)
+// index and the first hub index (U + 1 each), then the work
 __global__ void k_lv_totals(LevelArgs g, const int64_t* __restrict__ S, int64_t o_d, int64_t o_p,
-                            int64_t o_b, int64_t o_n, int64_t end, int64_t* __restrict__ out) {
+                            int64_t o_b, int64_t o_n, int64_t end, const Work* __restrict__ work,
+                            int64_t* __restrict__ out) {
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u == 0) {
     out[0] = S[o_d] - S[0];
     out[1] = S[o_b] - S[o_p];
     out[2] = S[end] - S[o_n];
+    int64_t* w = out + 3 + 2 * (g.n_units + 1);
+    w[0] = (int64_t)work->deg2;
+    w[1] = (int64_t)work->light_pairs;
+    w[2] = (int64_t)work->light_rows;
   }
   if (u > g.n_units) return;
   const int64_t e = g.n_units > 1 ? g.eseg[u] : (u ? g.n_edges : 0);
@@ -1936,7 +2011,71 @@ static size_t triples_smem(int theta) {
          (size_t)trip_slots(theta) * kTripSlot * 4;
 }
 
-static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
+// Do the levels take less time than what would count instead, the split kernels
+// or (kh-motifs) the scan?  Microseconds of each, from a first look at what
+// they go over, fitted on random hypergraphs of 60 to 400,000 hyperedges (a
+// first count, with its preparation; in ms, levels against split):
+//   * split, sparse rows: a pass over the pairs of each row's neighbours.
+//     250,000 hyperedges of 6 in communities of 200: 51 against 14; 400,000: 96
+//     against 23.
+//   * split, dense rows: a word scan a hyperwedge and 32 dense rows, where the
+//     cost model of tune.cu takes them; it is only asked when the sparse pass
+//     would win.  100,000 hyperedges in such communities: 13 against 51.
+//   * levels, light nodes: a look-up in the overlap matrix a pair of hyperedges
+//     at each light node pair, 7 ps, up to 27 where most rows are in a matrix
+//     past the caches; and at light nodes around rows of many heavy pairs, 20 and
+//     100 ps.  100,000 hyperedges of 10, all nodes of degree 100: 595 against
+//     413 where rows share many heavy pairs, 300 against 393 where they do not.
+//     This term is the least certain one (it does not know how often a look-up
+//     is repeated), so a lone hypergraph keeps the levels up to 1.3 times the
+//     other's time: 201,000 hyperedges of 6 in communities of 50, 187 against
+//     510, would else be on the wrong side, and the 595 stay there.
+//   * levels, matrix: clearing and mapping it, 0.2 us a MB.
+//   * levels, tables of classes: they grow with the square of the hyperedge
+//     size, and rows fill few of their entries.  1,500 uniform hyperedges of up
+//     to 60: 0.91 against 0.42; 300 Zipf ones, theta = 4: 0.68 against 0.58, and
+//     below 512 the levels are taken as they are (launches are most of both).
+//     In a batch a unit takes 9.3e-5 (entries x hyperedges)^0.65 against 0.015 a
+//     hyperedge and 1.2e-5 a squared line degree (up to 20,000 a hyperedge, from
+//     where dense rows pay), us: units of 60 hyperedges of up to 25, 6.7 against
+//     4.0 a unit, of 250 uniform ones 20 against 14, of 250 Zipf ones 19 against
+//     30, of 2,000 Zipf ones 111 against 481.
+//   * the scan, thresholds to 4 (levels against scan): 250,000 hyperedges in
+//     communities of 200 88 against 33, of 50 20 against 12; 6,000 uniform ones
+//     of up to 60 4.0 against 1.0; 4,001 Zipf ones 1.3 against 28.
+static int levels_pay(mochy_ctx* ctx, int theta, LevelsAgainst against, const Work& w,
+                      int64_t entries, size_t mat_bytes, int64_t n_dense, bool* pay) {
+  const double E = (double)ctx->n_edges, U = (double)ctx->n_units, deg2 = (double)w.deg2;
+  const bool lone = ctx->n_units == 1;
+  *pay = true;
+  if (lone && ctx->n_edges < 512 && against == LevelsAgainst::kSplit) return MOCHY_OK;
+  const double f = (double)n_dense / E;
+  const bool far = mat_bytes >= ((size_t)256 << 20);
+  double levels = 150.0 + 0.2e-6 * (double)mat_bytes;
+  if (lone || far)   // else in what a unit takes
+    levels += 1e-6 * 1024.0 * ((double)w.light_pairs * (7.0 + (far ? 20.0 * f * f : 0.0)) +
+                               (double)w.light_rows * (far ? 100.0 : 20.0));
+  levels += lone ? 3.7e-4 * (double)entries : U * 9.3e-5 * pow((double)entries * E / U, 0.65);
+  if (against == LevelsAgainst::kScan) {
+    *pay = levels * (theta + 3) / 4.0 <= 1.25 * (300.0 + 0.03 * E + 1e-5 * deg2);
+    return MOCHY_OK;
+  }
+  *pay = levels <= (lone ? 1.3 * (340.0 + 0.01 * E + 5e-6 * deg2)
+                         : 340.0 + 0.015 * E + 1.2e-5 * std::min(deg2, 2e4 * E));
+  if (*pay || !lone) return MOCHY_OK;
+  double sparse = 0.0, words = 0.0;
+  const int rc = model_split_work(ctx, &sparse, &words);
+  if (rc < 0) {
+    *pay = rc == MOCHY_E_UNSUPPORTED;   // the split kernels cannot count it
+    return *pay ? MOCHY_OK : rc;
+  }
+  *pay = levels <= 1.3 * (340.0 + 0.01 * E + 5e-6 * sparse + 2.5e-6 * words);
+  return MOCHY_OK;
+}
+
+// against: only when the levels take less time than that, else
+// MOCHY_E_UNSUPPORTED
+static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against) {
   cudaStream_t st = ctx->stream;
   const int64_t E = ctx->n_edges, N = ctx->n_nodes, T = ctx->n_inc;
   MOCHY_TRY(make_sides(ctx));
@@ -1967,7 +2106,7 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   const size_t b_scan = al((size_t)(n_seg + 1) * 8), b_ncls = al((size_t)N * Q * 4),
                b_hplus = al((size_t)E * 4), b_ehub = al((size_t)T * 2),
                b_unit = al((size_t)U * sizeof(LevelUnit)),
-               b_tot = al((size_t)(3 + 2 * (U + 1)) * 8);
+               b_tot = al((size_t)(3 + 2 * (U + 1) + 3) * 8);
   lv->bytes[0] = b_scan + b_ncls + 2 * b_hplus + b_ehub + b_unit + b_tot;
   MOCHY_TRY(dev_alloc(ctx, &lv->block[0], lv->bytes[0]));
   char* c = (char*)lv->block[0];
@@ -1980,19 +2119,27 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   int64_t* d_tot = (int64_t*)carve(b_tot);
   int32_t* many = (int32_t*)carve(b_hplus);
   void* t;
-  MOCHY_TRY(scratch(ctx, 0, (size_t)(n_seg + 1) * 8, &t));
+  MOCHY_TRY(scratch(ctx, 0, (size_t)(n_seg + 1) * 8 + sizeof(Work), &t));
   int64_t* seg = (int64_t*)t;
-  k_lv_rows<<<ceil_div(E, 256), 256, 0, st>>>(E, ctx->heavy_deg, ctx->esize, seg, seg + o_d,
-                                             seg + o_p);
+  Work* d_work = (Work*)(seg + n_seg + 1);
+  MOCHY_CUDA(cudaMemsetAsync(seg + n_seg, 0, 8 + sizeof(Work), st));
+  k_lv_rows<<<ceil_div(E, kRowThreads), kRowThreads, 0, st>>>(
+      E, ctx->noff, ctx->heavy_deg, ctx->esize, seg, seg + o_d, seg + o_p, d_work);
   MOCHY_LAUNCHED();
-  k_lv_nodes<<<row_grid(ctx, N, 8), kRowThreads, 0, st>>>(g, kHubDeg, ncls, seg + o_b, seg + o_n);
+  k_lv_nodes<<<row_grid(ctx, N, 8), kRowThreads, 0, st>>>(g, kHubDeg, ctx->heavy_deg, ncls, seg + o_b,
+                                                         seg + o_n, d_work);
   MOCHY_LAUNCHED();
-  MOCHY_CUDA(cudaMemsetAsync(seg + n_seg, 0, 8, st));
-  std::vector<int64_t> tot((size_t)3 + 2 * (U + 1));
+  std::vector<int64_t> tot((size_t)3 + 2 * (U + 1) + 3);
   const int64_t* hub_tot = tot.data() + 3 + U + 1;   // first hub of each unit
   for (bool ranked = false;; ranked = true) {
     MOCHY_TRY(scan_exclusive_i64(ctx, seg, scan, n_seg + 1));
-    k_lv_totals<<<ceil_div(U + 1, 128), 128, 0, st>>>(g, scan, o_d, o_p, o_b, o_n, n_seg, d_tot);
+    if (ranked) {
+      MOCHY_CUDA(cudaMemsetAsync(&d_work->light_pairs, 0, 16, st));
+      k_lv_light_work<<<ceil_div(E, kRowThreads), kRowThreads, 0, st>>>(g, ctx->heavy_deg, scan + o_b,
+                                                                       d_work);
+      MOCHY_LAUNCHED();
+    }
+    k_lv_totals<<<ceil_div(U + 1, 128), 128, 0, st>>>(g, scan, o_d, o_p, o_b, o_n, n_seg, d_work, d_tot);
     MOCHY_LAUNCHED();
     MOCHY_CUDA(cudaMemcpyAsync(tot.data(), d_tot, tot.size() * 8, cudaMemcpyDeviceToHost, st));
     MOCHY_CUDA(cudaStreamSynchronize(st));
@@ -2034,8 +2181,6 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
     un.hmoff = hub_pairs;
     hub_pairs += un.n_hubs * un.n_hubs;
   }
-  MOCHY_CUDA(cudaMemcpyAsync(d_unit, lv->units.data(), (size_t)U * sizeof(LevelUnit),
-                             cudaMemcpyHostToDevice, st));
   // 2. heavy rows, matrix, node pairs, tables
   g.tt = triple_table(theta);
   const int classes = trip_classes(theta);
@@ -2049,6 +2194,18 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   g.o_trip = g.o_out2 + n2;
   g.n_tab = g.o_trip + g.tt.total;
   g.tab_stride = (g.n_tab + 31) & ~(int64_t)31;
+  if (against != LevelsAgainst::kNothing) {
+    const int64_t* tw = tot.data() + 3 + 2 * (U + 1);
+    const Work w{(unsigned long long)tw[0], (unsigned long long)tw[1], (unsigned long long)tw[2]};
+    bool pay;
+    MOCHY_TRY(levels_pay(ctx, theta, against, w, g.n_tab, (size_t)mwords * 4, tot[3 + U], &pay));
+    if (!pay) {
+      ctx->levels_declined[(int)against] = theta;
+      return fail(MOCHY_E_UNSUPPORTED, "the levels take more time");
+    }
+  }
+  MOCHY_CUDA(cudaMemcpyAsync(d_unit, lv->units.data(), (size_t)U * sizeof(LevelUnit),
+                             cudaMemcpyHostToDevice, st));
   uint64_t slots = 64;
   while (slots < (uint64_t)(2 * P)) slots <<= 1;
   uint64_t oslots = 1 << 12;
@@ -2131,12 +2288,15 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta) {
   return MOCHY_OK;
 }
 
-int prepare_levels(mochy_ctx* ctx, int theta) {
+int prepare_levels(mochy_ctx* ctx, int theta, LevelsAgainst against) {
   if (ctx->levels && ctx->levels->ready && ctx->levels->theta == theta) return MOCHY_OK;
+  if (against != LevelsAgainst::kNothing &&
+      ctx->levels_declined[(int)against] == theta)   // of this line graph
+    return fail(MOCHY_E_UNSUPPORTED, "the levels take more time");
   release_levels(ctx);
   ctx->levels = new (std::nothrow) Levels();
   if (!ctx->levels) return fail(MOCHY_E_NOMEM, "host allocation failed");
-  const int rc = prepare(ctx, ctx->levels, theta);
+  const int rc = prepare(ctx, ctx->levels, theta, against);
   if (rc < 0) release_levels(ctx);
   return rc;
 }

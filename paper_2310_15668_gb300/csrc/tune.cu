@@ -27,7 +27,9 @@ namespace mochy {
 size_t dense_smem_bytes(int64_t W);       // count_split.cu
 size_t sparse_smem_bytes(int max_deg);    // count_split.cu
 
+// The model's threshold, kept with the line graph.
 int choose_dense_threshold(mochy_ctx* ctx) {
+  if (ctx->model_thr > 0) return ctx->model_thr;
   const int64_t E = ctx->n_edges;
   std::vector<int64_t> off((size_t)E + 1);
   MOCHY_CUDA(cudaMemcpyAsync(off.data(), ctx->noff, off.size() * 8, cudaMemcpyDeviceToHost,
@@ -46,10 +48,10 @@ int choose_dense_threshold(mochy_ctx* ctx) {
     }
   const double word_weight = 0.1;
   int best = -1;
-  double best_cost = 0.0;
+  double best_cost = 0.0, best_sparse = 0.0, best_words = 0.0;
   for (int64_t thr = 32; thr <= (int64_t)1 << 20; thr <<= 1) {
     int64_t nd_all = 0, max_sparse = 0, wmax = 1;
-    double cost = 0.0;
+    double cost = 0.0, sparse_all = 0.0, words = 0.0;
     for (int u = 0; u < U; ++u) {
       int64_t nd = 0;
       double Sd = 0.0, sparse = 0.0;
@@ -66,6 +68,8 @@ int choose_dense_threshold(mochy_ctx* ctx) {
       wmax = std::max(wmax, U > 1 ? W + 1 : W);   // a unit's window may straddle a word
       const double fd = S[u] > 0 ? Sd / S[u] : 0.0;
       cost += word_weight * 0.5 * Sd * fd * (double)W / 3.0 + sparse;
+      sparse_all += sparse;
+      words += 0.5 * Sd * fd * (double)W;
       nd_all += nd;
     }
     if (dense_smem_bytes(wmax) + 1024 > ctx->smem_optin) continue;
@@ -74,11 +78,27 @@ int choose_dense_threshold(mochy_ctx* ctx) {
     if (best < 0 || cost < best_cost) {
       best = (int)thr;
       best_cost = cost;
+      best_sparse = sparse_all;
+      best_words = words;
     }
     if (nd_all == 0) break;   // larger thresholds change nothing
   }
   if (best < 0) return fail(MOCHY_E_UNSUPPORTED, "no dense threshold fits shared memory");
+  ctx->model_thr = best;
+  ctx->model_sparse = best_sparse;
+  ctx->model_words = best_words;
   return best;
+}
+
+// What the split kernels have to go over at the model's threshold: pairs of
+// neighbours of sparse rows, words scanned for dense ones (all of them, where
+// the model's weight is on the few that matter).
+int model_split_work(mochy_ctx* ctx, double* sparse, double* words) {
+  const int thr = choose_dense_threshold(ctx);
+  if (thr < 0) return thr;
+  *sparse = ctx->model_sparse;
+  *words = ctx->model_words;
+  return MOCHY_OK;
 }
 
 }  // namespace mochy

@@ -137,3 +137,65 @@ def test_hubs_of_crowded_units_in_a_batch():
     got = B.mochy_profile_batch(gs, 1, seeds)
     ref = B.mochy_profile_batch(gs, 1, seeds, cfg)
     assert np.array_equal(got[4], ref[4]) and np.array_equal(got[5], ref[5])
+
+
+def _communities(edges, group, size, mult, seed):
+    """`edges` hyperedges within communities of `group` nodes, mult * group
+    drawn in each: nearly every one shares two nodes with some others, and
+    line-graph rows are short."""
+    rng = np.random.default_rng(seed)
+    g = rng.integers(0, max(1, edges // (mult * group)), int(edges * 1.1) + 10)
+    m = np.sort(g[:, None] * group + rng.integers(0, group, (len(g), size)), 1)
+    m = np.unique(m[(np.diff(m, axis=1) > 0).all(1)], axis=0)
+    m = m[rng.permutation(len(m))[:edges]]
+    n = (max(1, edges // (mult * group))) * group
+    return n, np.arange(len(m) + 1, dtype=np.int64) * size, m.astype(np.int32).ravel()
+
+
+def _route(g, **kw):
+    """Counts, and whether the levels made them."""
+    with B.Context(**kw) as c:
+        c.load(*g)
+        c.project()
+        B.mochy_trace(c.h, 1)
+        got = c.count_exact()
+        return got, "level 3" in B.mochy_trace_read(c.h)["phases_ms"]
+
+
+@pytest.mark.parametrize("g,theta,levels", [
+    ((110000, 50, 4, 3, 61), 1, False),      # sparse rows: an overlap matrix of 5 GB for few pairs
+    ((6000, 1000, 10, 6, 62), 1, True),      # longer rows
+    ((6000, 1000, 3, 6, 63), 3, True),
+])
+def test_sparse_hypergraphs_are_left_to_the_split_kernels(g, theta, levels):
+    g = _communities(*g)
+    (h, h3), by_levels = _route(g, theta=theta)
+    oh, o3 = _count(g, theta=theta, rest_path=2)      # the split kernels
+    assert np.array_equal(h, oh) and np.array_equal(h3, o3)
+    assert by_levels == levels
+
+
+@pytest.mark.parametrize("units,nodes,edges,most,levels", [(300, 200, 50, 12, False),
+                                                           (12, 900, 900, 6, True)])
+def test_batches_of_small_hypergraphs_are_left_to_the_split_kernels(units, nodes, edges, most,
+                                                                     levels):
+    kinds = [_wide(nodes, edges, 2, most, 700 + q) for q in range(4)]
+    gs = [kinds[q % 4] for q in range(units)]
+    seeds = list(range(units))
+    _, _, _, _, ch, c3, _, info = B.mochy_profile_batch(gs, 3, seeds)
+    for g in range(4):
+        o = oracle.profile(*gs[g], 3, seeds[g])
+        assert np.array_equal(ch[g], o["counts_h"]) and np.array_equal(c3[g], o["counts_3h"])
+    assert (info["dense_threshold"] == 0) == levels
+
+
+@pytest.mark.parametrize("theta", [1, 4])
+def test_kh_motifs_of_a_sparse_hypergraph(theta):
+    """k = 3 is the 3h-motifs, whichever of levels, scan and split counts."""
+    g = _communities(110000, 50, 4, 3, 64)
+    with B.Context(theta=theta) as c:
+        c.load(*g)
+        c.project()
+        h, h3 = c.count_exact()
+        kh, k3 = c.count_kh(3, (theta,))
+    assert np.array_equal(h, kh) and np.array_equal(h3, k3)

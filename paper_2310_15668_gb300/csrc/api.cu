@@ -162,15 +162,20 @@ void dev_free(mochy_ctx* ctx, void* p, size_t bytes) {
   }
 }
 
+int drop_scratch(mochy_ctx* ctx, int slot) {
+  Buffer& b = ctx->scratch[slot];
+  if (!b.p) return MOCHY_OK;
+  MOCHY_CUDA(cudaStreamSynchronize(ctx->stream));
+  dev_free(ctx, b.p, b.bytes);
+  b.p = nullptr;
+  b.bytes = 0;
+  return MOCHY_OK;
+}
+
 int scratch(mochy_ctx* ctx, int slot, size_t bytes, void** p) {
   Buffer& b = ctx->scratch[slot];
   if (b.bytes < bytes) {
-    if (b.p) {
-      MOCHY_CUDA(cudaStreamSynchronize(ctx->stream));
-      dev_free(ctx, b.p, b.bytes);
-      b.p = nullptr;
-      b.bytes = 0;
-    }
+    MOCHY_TRY(drop_scratch(ctx, slot));
     const size_t grow = bytes + bytes / 4 + 4096;
     MOCHY_TRY(dev_alloc(ctx, &b.p, grow));
     b.bytes = grow;

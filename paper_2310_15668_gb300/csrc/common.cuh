@@ -237,6 +237,7 @@ int ensure_dynamic_smem(const void* func, size_t bytes);
 int dev_alloc(mochy_ctx* ctx, void** p, size_t bytes);
 void dev_free(mochy_ctx* ctx, void* p, size_t bytes);
 int scratch(mochy_ctx* ctx, int slot, size_t bytes, void** p);
+int drop_scratch(mochy_ctx* ctx, int slot);   // gives one slot's block up
 void release_graph(mochy_ctx* ctx);
 void release_projection(mochy_ctx* ctx);
 

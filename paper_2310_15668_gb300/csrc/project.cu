@@ -82,7 +82,8 @@ k_project_bitmaps(ProjArgs g, unsigned long long* __restrict__ cursor) {
   }
 }
 
-template <bool FILL>
+// BITS: some node may have a bitmap
+template <bool FILL, bool BITS>
 __global__ void __launch_bounds__(kProjThreads) k_project_rows(ProjArgs g) {
   __shared__ uint2 s_word[kProjWarps][32];      // neighbour bits, entries before the word
   __shared__ uint32_t s_twice[kProjWarps][32];  // ids met twice or more
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(kProjThreads) k_project_rows(ProjArgs g) {
         const int32_t v = g.enode[eb + p];
         cur[s] = g.voff[v];
         last[s] = g.voff[v + 1];
-        bm[s] = g.bitmap[v];
+        if (BITS) bm[s] = g.bitmap[v];
         if (bm[s] < 0) next[s] = g.vedge[cur[s]];
       }
       hubs[s] = __ballot_sync(0xffffffffu, bm[s] >= 0);
@@ -322,10 +323,14 @@ int project_graph(mochy_ctx* ctx) {
   int64_t* below = deg + (E + 1);
   int64_t* uplen = below + (E + 1);
   MOCHY_CUDA(cudaMemsetAsync(deg, 0, (size_t)(E + 1) * 8 * 3, st));
-  // bitmaps of the nodes of high degree (at most 9 words per incidence)
+  // Bitmaps of the nodes of high degree (at most 9 words per incidence).  The
+  // rows come out the same without them, so they do not take memory that the
+  // line graph needs.
   const size_t b_nodes = (size_t)ctx->n_nodes * 8, b_bits = (size_t)ctx->n_inc * 36 + 256;
-  void* t2;
-  MOCHY_TRY(scratch(ctx, 2, b_nodes + 8 + b_bits, &t2));
+  void* t2 = nullptr;
+  const int rc2 = scratch(ctx, 2, b_nodes + 8 + b_bits, &t2);
+  if (rc2 < 0 && rc2 != MOCHY_E_NOMEM) return rc2;
+  if (rc2 < 0) t2 = nullptr;
   ProjArgs g;
   g.n_edges = E;
   g.n_nodes = ctx->n_nodes;
@@ -338,20 +343,23 @@ int project_graph(mochy_ctx* ctx) {
   g.nseg = ctx->d_nseg;
   g.eseg = ctx->d_nseg ? ctx->d_nseg + ctx->n_units + 1 : nullptr;
   g.bitmap = (int64_t*)t2;
-  g.bits = (uint32_t*)((char*)t2 + b_nodes + 8);
+  g.bits = t2 ? (uint32_t*)((char*)t2 + b_nodes + 8) : nullptr;
   g.deg = deg;
   g.below = below;
   g.heavy = ctx->heavy_deg;
   g.noff = ctx->noff;
   g.nadj = nullptr;
-  MOCHY_CUDA(cudaMemsetAsync((char*)t2 + b_nodes, 0, 8 + b_bits, st));
-  k_project_bitmaps<<<(unsigned)std::min<int64_t>(ceil_div(ctx->n_nodes, 8),
-                                                 (int64_t)ctx->num_sms * 8),
-                      256, 0, st>>>(g, (unsigned long long*)((char*)t2 + b_nodes));
-  MOCHY_LAUNCHED();
+  if (t2) {
+    MOCHY_CUDA(cudaMemsetAsync((char*)t2 + b_nodes, 0, 8 + b_bits, st));
+    k_project_bitmaps<<<(unsigned)std::min<int64_t>(ceil_div(ctx->n_nodes, 8),
+                                                   (int64_t)ctx->num_sms * 8),
+                        256, 0, st>>>(g, (unsigned long long*)((char*)t2 + b_nodes));
+    MOCHY_LAUNCHED();
+  }
   const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(E, kProjWarps),
                                                     (int64_t)ctx->num_sms * 16);
-  k_project_rows<false><<<grid, kProjThreads, 0, st>>>(g);
+  auto lengths = t2 ? k_project_rows<false, true> : k_project_rows<false, false>;
+  lengths<<<grid, kProjThreads, 0, st>>>(g);
   MOCHY_LAUNCHED();
   MOCHY_TRY(scan_exclusive_i64(ctx, deg, ctx->noff, E + 1));
   int64_t total = 0;
@@ -359,6 +367,11 @@ int project_graph(mochy_ctx* ctx) {
   MOCHY_CUDA(cudaStreamSynchronize(st));
   const size_t bytes = (size_t)std::max<int64_t>(total, 1) * sizeof(uint2);
   int rc = dev_alloc(ctx, &p, bytes);
+  if (rc == MOCHY_E_NOMEM && t2) {
+    MOCHY_TRY(drop_scratch(ctx, 2));
+    t2 = nullptr;
+    rc = dev_alloc(ctx, &p, bytes);
+  }
   if (rc < 0) {
     release_projection(ctx);
     return fail(MOCHY_E_NOMEM, "line graph needs " + std::to_string(bytes) +
@@ -366,9 +379,9 @@ int project_graph(mochy_ctx* ctx) {
   }
   ctx->nadj = (uint2*)p;
   g.nadj = ctx->nadj;
-  k_project_rows<true><<<(unsigned)std::min<int64_t>(ceil_div(E, kProjWarps),
-                                                     (int64_t)ctx->num_sms * 8),
-                         kProjThreads, 0, st>>>(g);
+  auto entries = t2 ? k_project_rows<true, true> : k_project_rows<true, false>;
+  entries<<<(unsigned)std::min<int64_t>(ceil_div(E, kProjWarps), (int64_t)ctx->num_sms * 8),
+            kProjThreads, 0, st>>>(g);
   MOCHY_LAUNCHED();
   int* maxdeg = ctx->counters + 2;
   MOCHY_CUDA(cudaMemsetAsync(maxdeg, 0, 4, st));
@@ -381,6 +394,7 @@ int project_graph(mochy_ctx* ctx) {
   ctx->n_wedges = total / 2;
   ctx->max_deg = md;
   ctx->projected = true;
+  if (ctx->budget > 0) MOCHY_TRY(drop_scratch(ctx, 2));   // a budget counts what is held
   return MOCHY_OK;
 }
 

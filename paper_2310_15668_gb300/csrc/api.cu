@@ -78,6 +78,8 @@ void give_back(mochy_ctx* ctx) {
 
 }  // namespace
 
+static int dev_alloc_once(mochy_ctx* ctx, void** p, size_t bytes);
+
 void keep_blocks(mochy_ctx* ctx) {
   std::lock_guard<std::mutex> lk(kept_mu);
   ctx->kept_max = kKeptBytes;
@@ -92,7 +94,18 @@ void keep_no_blocks(mochy_ctx* ctx) {
                       kept_contexts.end());
 }
 
+// An allocation that the budget or the device refuses is tried once more without
+// the level structures, when these are complete: they are kept between counts,
+// are built again by the next one or replaced by the split kernels', and must
+// not make a call fail that does not need them.
 int dev_alloc(mochy_ctx* ctx, void** p, size_t bytes) {
+  const int rc = dev_alloc_once(ctx, p, bytes);
+  if (rc != MOCHY_E_NOMEM || !levels_kept(ctx)) return rc;
+  release_levels(ctx);
+  return dev_alloc_once(ctx, p, bytes);
+}
+
+static int dev_alloc_once(mochy_ctx* ctx, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
   if (ctx->budget > 0 && ctx->held + (int64_t)bytes > ctx->budget)

@@ -238,6 +238,7 @@ int dev_alloc(mochy_ctx* ctx, void** p, size_t bytes);
 void dev_free(mochy_ctx* ctx, void* p, size_t bytes);
 int scratch(mochy_ctx* ctx, int slot, size_t bytes, void** p);
 int drop_scratch(mochy_ctx* ctx, int slot);   // gives one slot's block up
+void release_scratch(mochy_ctx* ctx);         // all of them
 void release_graph(mochy_ctx* ctx);
 void release_projection(mochy_ctx* ctx);
 
@@ -274,6 +275,7 @@ struct PhaseTimer;
 int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const uint16_t* lut, int k,
                   int t1, int t2, PhaseTimer* timer);                 // levels.cu
 void release_levels(mochy_ctx* ctx);                                  // levels.cu
+bool levels_kept(const mochy_ctx* ctx);                               // levels.cu
 int prepare_exact(mochy_ctx* ctx, bool* by_levels);                   // count_split.cu
 int choose_dense_threshold(mochy_ctx* ctx);                           // tune.cu
 int model_split_work(mochy_ctx* ctx, double* sparse, double* words);  // tune.cu

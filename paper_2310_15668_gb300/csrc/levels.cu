@@ -1971,6 +1971,10 @@ void release_levels(mochy_ctx* ctx) {
   delete lv;
 }
 
+// complete structures, in no call's use: none allocates between preparing the
+// levels and launching their kernels, and release_levels waits for these
+bool levels_kept(const mochy_ctx* ctx) { return ctx->levels && ctx->levels->ready; }
+
 bool levels_cover(int theta, int64_t n_edges, int n_units) {
   // a tuple key has 19 bits left for the unit
   return theta <= kMaxTheta && n_edges > 0 && n_units < (1 << 18);
@@ -2078,6 +2082,7 @@ static int levels_pay(mochy_ctx* ctx, int theta, LevelsAgainst against, const Wo
 static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against) {
   cudaStream_t st = ctx->stream;
   const int64_t E = ctx->n_edges, N = ctx->n_nodes, T = ctx->n_inc;
+  if (!ctx->heavy_deg) return fail(MOCHY_E_NOMEM, "its memory holds the row order");
   MOCHY_TRY(make_sides(ctx));
   const int U = ctx->n_units, Q = theta + 3, S = std::max(ctx->max_size, 2);
   LevelArgs& g = lv->g;
@@ -2298,6 +2303,8 @@ int prepare_levels(mochy_ctx* ctx, int theta, LevelsAgainst against) {
   if (!ctx->levels) return fail(MOCHY_E_NOMEM, "host allocation failed");
   const int rc = prepare(ctx, ctx->levels, theta, against);
   if (rc < 0) release_levels(ctx);
+  // a budget counts what is held: the preparation's scratch is not kept there
+  if (ctx->budget > 0) release_scratch(ctx);
   return rc;
 }
 

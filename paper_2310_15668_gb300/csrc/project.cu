@@ -420,7 +420,16 @@ int ensure_row_order(mochy_ctx* ctx) {
     MOCHY_TRY(radix_sort_pairs_u32(ctx, key, val, E, bits_for(ctx->n_units)));
   }
   void* p;
-  MOCHY_TRY(dev_alloc(ctx, &p, sizeof(int32_t) * (size_t)E));
+  const int rc = dev_alloc(ctx, &p, sizeof(int32_t) * (size_t)E);
+  if (rc == MOCHY_E_NOMEM && ctx->heavy_deg) {
+    // no room for both: the order takes the place of the heavy degrees, which
+    // only the levels read
+    release_levels(ctx);
+    p = ctx->heavy_deg;
+    ctx->heavy_deg = nullptr;
+  } else if (rc < 0) {
+    return rc;
+  }
   ctx->row_order = (int32_t*)p;
   MOCHY_CUDA(cudaMemcpyAsync(ctx->row_order, val, (size_t)E * 4, cudaMemcpyDeviceToDevice, st));
   return MOCHY_OK;

@@ -28,7 +28,6 @@ namespace mochy {
 
 int64_t estimate_graph_bytes(int64_t n_nodes, int64_t n_edges, const int64_t* off,
                              const int32_t* nodes);   // batch.cu
-void release_scratch(mochy_ctx* ctx);                 // api.cu
 void keep_no_blocks(mochy_ctx* ctx);                  // api.cu
 
 namespace {

@@ -74,3 +74,25 @@ def test_projection_needs_the_line_graph_alone(spec):
     calls = [_load(g), _project, lambda c: c.count_sampled(B.MOCHY_A_PLUS, 300, 5)]
     for a, b in zip(_fits(need + (1 << 20), calls)[2], _fits(1 << 32, calls)[2]):
         assert np.array_equal(a, b)
+
+
+def _exact(c):
+    return c.count_exact()
+
+
+def _profiles(c):
+    return c.hyperedge_profile()
+
+
+@pytest.mark.parametrize("spec", [SPEC, FLAT])
+@pytest.mark.parametrize("after", [(), (_profiles,), (lambda c: c.count_kh(2, ()),)])
+def test_exact_counts_fit_where_the_split_kernels_do(spec, after):
+    """The level structures are taken where there is room for them, and given
+    up for a later call that needs it."""
+    calls = [_load(_graph(spec)), _project, _exact, *after]
+    with_levels, got = _least(calls)
+    split, ref = _least(calls, rest_path=2)
+    assert with_levels <= split
+    for a, b in zip(got[2:], ref[2:]):
+        for x, y in zip(a, b):
+            assert np.array_equal(x, y)

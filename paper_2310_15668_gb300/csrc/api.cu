@@ -821,6 +821,8 @@ int mochy_count_sampled(mochy_ctx* ctx, int method, int64_t samples, uint64_t se
   int64_t* h = (int64_t*)ctx->pinned;
   MOCHY_CUDA(cudaMemcpyAsync(h, d_counts, 457 * 16, cudaMemcpyDeviceToHost, ctx->stream));
   MOCHY_CUDA(cudaStreamSynchronize(ctx->stream));
+  // a budget counts what is held: the rows' class histograms and the draws are not
+  if (ctx->budget > 0) release_scratch(ctx);
   const double* he = (const double*)(h + 457);
   if (raw_h) memcpy(raw_h, h, MOCHY_N_H * 8);
   if (raw_3h) memcpy(raw_3h, h + MOCHY_N_H, MOCHY_N_3H * 8);

@@ -96,3 +96,17 @@ def test_exact_counts_fit_where_the_split_kernels_do(spec, after):
     for a, b in zip(got[2:], ref[2:]):
         for x, y in zip(a, b):
             assert np.array_equal(x, y)
+
+
+def test_sampling_leaves_its_room_to_later_calls():
+    """Class histograms and grouped draws of long rows are scratch of the call."""
+    g = _graph(SPEC)
+    assert 2 * 1462159 >= 256 * (len(g[1]) - 1)          # long enough rows for both methods
+    samples = [lambda c: c.count_sampled(B.MOCHY_A, 300, 3),
+               lambda c: c.count_sampled(B.MOCHY_A_PLUS, 9000, 4)]
+    without, _ = _least([_load(g), _project, _profiles])
+    sampled, got = _least([_load(g), _project, *samples, _profiles])
+    assert sampled <= without
+    for a, b in zip(got[2:4], _fits(1 << 32, [_load(g), _project, *samples])[2:]):
+        for x, y in zip(a, b):
+            assert np.array_equal(x, y)

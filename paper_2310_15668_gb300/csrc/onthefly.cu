@@ -12,8 +12,8 @@
 //   * the sorted incidence lists E_v of the other nodes, merged into the
 //     scan chunk by chunk.
 // Three uses of the scan:
-//   1. degrees: d_i = |N_{e_i}| and the number of neighbours after i (the
-//      ascending (i, j) order of hyperwedges that MoCHy-A+ draws from);
+//   1. the number of neighbours after each hyperedge i (the ascending (i, j)
+//      order of hyperwedges that MoCHy-A+ draws from);
 //   2. the draw: hyperwedge n is index floor(u |wedges| / 2^64) of that
 //      order, as for the projected MoCHy-A+, so e_j is the o-th neighbour of
 //      e_i after i, found by popcounts along the scan;
@@ -60,8 +60,7 @@ struct OtfArgs {
   uint64_t seed;
   int64_t samples;
   int32_t* queue;
-  int64_t* deg;                   // degree pass: d_i and neighbours after i
-  int64_t* up;
+  int64_t* up;                    // degree pass: the neighbours after i
   unsigned long long* stats;      // [4] candidates, words scanned, list entries, exact
   // the draws and the bitmaps in order of size (k_otf_draw, k_otf_classify)
   int64_t first, n_draws, n_seg;  // this launch's draws, parts of a draw's scan
@@ -258,8 +257,8 @@ __device__ __forceinline__ uint32_t any_of(const Slices& s, int p) {
   return s.c[p][0] | s.c[p][1] | s.c[p][2] | s.c[p][3];
 }
 
-// Degrees: one warp per hyperedge e_i; its neighbours are the hyperedges
-// marked in the union over its nodes, except i itself.
+// Neighbours after each hyperedge: one warp per e_i; they are the hyperedges
+// marked after i in the union over its nodes.
 __global__ void __launch_bounds__(kOtfThreads) k_otf_degrees(OtfArgs g) {
   extern __shared__ __align__(16) unsigned char smem[];
   OtfWarp& me = ((OtfWarp*)smem)[threadIdx.x >> 5];
@@ -274,28 +273,20 @@ __global__ void __launch_bounds__(kOtfThreads) k_otf_degrees(OtfArgs g) {
     if (lane + 32 < A) me.anodes[lane + 32] = g.enode[g.eoff[i] + lane + 32];
     __syncwarp();
     split_nodes(g, me, A, 0, false, 0);
-    unsigned long long d = 0, u = 0, ent = 0;
+    unsigned long long u = 0, ent = 0;
     const bool scan_all = me.nh > 0;
     int64_t w0 = scan_all ? 0 : next_list_word(g, me);
     while (w0 < g.W) {
       Slices s;
       gather_chunk(g, me, w0, s, ent);
       const int64_t w = w0 + lane;
-      uint32_t m = w < g.W ? any_of(s, 0) : 0u;
-      if (w == (i >> 5)) m &= ~(1u << (i & 31));
-      d += __popc(m);
+      const uint32_t m = w < g.W ? any_of(s, 0) : 0u;
       if (w > (i >> 5)) u += __popc(m);
       else if (w == (i >> 5) && (i & 31) != 31) u += __popc(m & (0xffffffffu << ((i & 31) + 1)));
       w0 = scan_all ? w0 + 32 : max(w0 + 32, next_list_word(g, me));
     }
-    for (int dd = 16; dd; dd >>= 1) {
-      d += __shfl_xor_sync(0xffffffffu, d, dd);
-      u += __shfl_xor_sync(0xffffffffu, u, dd);
-    }
-    if (lane == 0) {
-      g.deg[i] = (int64_t)d;
-      g.up[i] = (int64_t)u;
-    }
+    for (int dd = 16; dd; dd >>= 1) u += __shfl_xor_sync(0xffffffffu, u, dd);
+    if (lane == 0) g.up[i] = (int64_t)u;
     __syncwarp();
   }
 }
@@ -1270,36 +1261,44 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
   std::sort(pop.begin(), pop.end());
   const int64_t cap_bytes =
       budget > 0 ? budget : (ctx->budget > 0 ? ctx->budget / 4 : ((int64_t)4 << 30));
-  const int64_t max_bitmaps = std::min<int64_t>((int64_t)pop.size(), cap_bytes / (W * 4));
+  int64_t max_bitmaps = std::min<int64_t>((int64_t)pop.size(), cap_bytes / (W * 4));
+  auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  // bitmaps in order of size as well when all of both fit the budget; each of
+  // the 64 sizes begins on four words
+  const int64_t Wp = W + 4 * kOtfSizes;
+  bool by_size = max_bitmaps == (int64_t)pop.size() &&
+                 (int64_t)pop.size() * (W + Wp) * 4 <= cap_bytes;
+  const size_t b_hidx = al((size_t)std::max<int64_t>(N, 1) * 4);
+  const size_t b_sbits = al((size_t)4 * W * 4);
+  const size_t b_pre = al((size_t)(E + 1) * 8);
+  const size_t b_pos = al((size_t)std::max<int64_t>(E, 1) * 4), b_id = al((size_t)Wp * 32 * 4);
+  size_t b_nodes, b_one, b_bits, b_order, b_up, bytes;
+  void* p = nullptr;
+  // What makes the call faster takes only the memory that there is: without
+  // room for both sets of bitmaps one is left out, then the least popular
+  // nodes' bitmaps.
+  while (true) {
+    b_nodes = al((size_t)std::max<int64_t>(max_bitmaps, 1) * 4);
+    b_one = al((size_t)std::max<int64_t>(max_bitmaps, 1) * W * 4);
+    b_bits = by_size ? b_one + al((size_t)std::max<int64_t>(max_bitmaps, 1) * Wp * 4) : b_one;
+    // by size: the positions (both ways) and the sizes' first words; the draws
+    // of a launch take the place of the neighbours after each hyperedge once
+    // these are summed (E + 1 entries: the scan reads them all)
+    b_order = by_size ? b_pos + b_id + al((2 * kOtfSizes + 1) * 4) : 0;
+    b_up = al((size_t)(E + 1) * 8);
+    if (by_size) b_up = std::max(b_up, kOtfDrawBytes);
+    bytes = b_hidx + b_nodes + b_bits + b_sbits + b_pre + b_order + b_up;
+    const int rc = dev_alloc(ctx, &p, bytes);
+    if (rc == MOCHY_OK) break;
+    if (rc != MOCHY_E_NOMEM || (!by_size && max_bitmaps == 0)) return rc;
+    if (by_size) by_size = false;
+    else max_bitmaps = max_bitmaps * 3 / 4;
+  }
   std::vector<int32_t> hidx((size_t)N, -1), nodes_of((size_t)std::max<int64_t>(max_bitmaps, 1), 0);
   for (int64_t h = 0; h < max_bitmaps; ++h) {
     hidx[(size_t)pop[h].second] = (int32_t)h;
     nodes_of[(size_t)h] = pop[h].second;
   }
-  auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const size_t b_hidx = al((size_t)std::max<int64_t>(N, 1) * 4);
-  const size_t b_nodes = al(nodes_of.size() * 4);
-  // bitmaps in order of size as well when all of both fit the budget; each of
-  // the 64 sizes begins on four words
-  const int64_t Wp = W + 4 * kOtfSizes;
-  const bool by_size = max_bitmaps == (int64_t)pop.size() &&
-                       (int64_t)pop.size() * (W + Wp) * 4 <= cap_bytes;
-  const size_t b_one = al((size_t)std::max<int64_t>(max_bitmaps, 1) * W * 4);
-  const size_t b_bits = by_size ? b_one + al((size_t)std::max<int64_t>(max_bitmaps, 1) * Wp * 4)
-                                : b_one;
-  const size_t b_sbits = al((size_t)4 * W * 4);
-  const size_t b_pre = al((size_t)(E + 1) * 8);
-  // by size: the positions (both ways) and the sizes' first words take the
-  // place of the degrees, and the draws of a launch that of the neighbours
-  // after i, once these are summed
-  const size_t b_pos = al((size_t)std::max<int64_t>(E, 1) * 4), b_id = al((size_t)Wp * 32 * 4);
-  const size_t b_deg = by_size ? b_pos + b_id + al((2 * kOtfSizes + 1) * 4)
-                               : al((size_t)std::max<int64_t>(E, 1) * 8);
-  // E + 1 entries: the scan reads them all (the last only lends its place)
-  const size_t b_up = std::max(al((size_t)(E + 1) * 8), kOtfDrawBytes);
-  const size_t bytes = b_hidx + b_nodes + b_bits + b_sbits + b_pre + b_deg + b_up;
-  void* p = nullptr;
-  MOCHY_TRY(dev_alloc(ctx, &p, bytes));
   char* c = (char*)p;
   ctx->otf_block = p;
   ctx->otf_bytes = bytes;
@@ -1308,8 +1307,8 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
   ctx->otf_hbits = (uint32_t*)(c + b_hidx + b_nodes);
   ctx->otf_sbits = (uint32_t*)(c + b_hidx + b_nodes + b_bits);
   ctx->otf_uprefix = (int64_t*)(c + b_hidx + b_nodes + b_bits + b_sbits);
-  int64_t* deg = (int64_t*)(c + b_hidx + b_nodes + b_bits + b_sbits + b_pre);
-  int64_t* up = (int64_t*)((char*)deg + b_deg);
+  int32_t* pos_of = (int32_t*)(c + b_hidx + b_nodes + b_bits + b_sbits + b_pre);
+  int64_t* up = (int64_t*)((char*)pos_of + b_order);
   auto bail = [&](int rc) { release_onthefly(ctx); return rc; };
   if (cudaMemcpyAsync(ctx->otf_hidx, hidx.data(), (size_t)N * 4, cudaMemcpyHostToDevice, st) !=
           cudaSuccess ||
@@ -1321,8 +1320,8 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
   if (by_size) {
     ctx->otf_pwords = Wp;
     ctx->otf_pbits = (uint32_t*)((char*)ctx->otf_hbits + b_one);
-    ctx->otf_id_of = (int32_t*)((char*)deg + b_pos);
-    ctx->otf_cls = (int32_t*)((char*)deg + b_pos + b_id);
+    ctx->otf_id_of = (int32_t*)((char*)pos_of + b_pos);
+    ctx->otf_cls = (int32_t*)((char*)pos_of + b_pos + b_id);
     ctx->otf_draws = up;
     ctx->otf_max_draws = (int64_t)(b_up / 8);
     int32_t* counts = ctx->otf_cls + kOtfSizes + 1;
@@ -1333,7 +1332,7 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
                     st>>>(E, ctx->esize, counts);
       k_otf_starts<<<1, 32, 0, st>>>(counts, ctx->otf_cls);
       k_otf_positions<<<(unsigned)ceil_div(E, 256), 256, 0, st>>>(E, ctx->esize, counts,
-                                                                 (int32_t*)deg, ctx->otf_id_of);
+                                                                 pos_of, ctx->otf_id_of);
       note_launch();
       note_launch();
       note_launch();
@@ -1341,7 +1340,7 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
   }
   if (max_bitmaps > 0) {
     k_otf_bits<<<(unsigned)std::min<int64_t>(max_bitmaps, 4096), 256, 0, st>>>(
-        max_bitmaps, W, d_nodes_of, ctx->voff, ctx->vedge, ctx->otf_hbits, Wp, (int32_t*)deg,
+        max_bitmaps, W, d_nodes_of, ctx->voff, ctx->vedge, ctx->otf_hbits, Wp, pos_of,
         by_size ? ctx->otf_pbits : nullptr);
     note_launch();
   }
@@ -1360,7 +1359,6 @@ int prepare_onthefly(mochy_ctx* ctx, int64_t budget) {
   g.hidx = ctx->otf_hidx;
   g.hbits = ctx->otf_hbits;
   g.sbits = ctx->otf_sbits;
-  g.deg = deg;
   g.up = up;
   if (E > 0 && max_bitmaps == (int64_t)pop.size()) {
     k_otf_after<<<(unsigned)std::min<int64_t>(ceil_div(E, kAfterThreads / 32),

@@ -185,11 +185,18 @@ int drop_scratch(mochy_ctx* ctx, int slot) {
   return MOCHY_OK;
 }
 
+static size_t scratch_size(size_t bytes) { return bytes + bytes / 4 + 4096; }
+
+size_t scratch_growth(const mochy_ctx* ctx, int slot, size_t bytes) {
+  const Buffer& b = ctx->scratch[slot];
+  return b.bytes < bytes ? scratch_size(bytes) - b.bytes : 0;
+}
+
 int scratch(mochy_ctx* ctx, int slot, size_t bytes, void** p) {
   Buffer& b = ctx->scratch[slot];
   if (b.bytes < bytes) {
     MOCHY_TRY(drop_scratch(ctx, slot));
-    const size_t grow = bytes + bytes / 4 + 4096;
+    const size_t grow = scratch_size(bytes);
     MOCHY_TRY(dev_alloc(ctx, &b.p, grow));
     b.bytes = grow;
   }
@@ -884,6 +891,7 @@ int mochy_profile(mochy_ctx* ctx, int32_t n_random, uint64_t seed, double* sig_h
   ctx->copies = nullptr;
   if (rc == MOCHY_OK && !copy_ctx) rc = new_like(ctx, &copy_ctx);
   if (rc == MOCHY_OK && ctx->kept_max == 0) keep_no_blocks(copy_ctx);
+  if (rc == MOCHY_OK) copy_ctx->reserved = ctx->reserved;
   for (int32_t c = 0; rc == MOCHY_OK && c < n_random; ++c) {
     rc = randomize_graph(ctx, seed, (uint32_t)c, copy_ctx);
     if (rc == MOCHY_OK) rc = project_graph(copy_ctx);

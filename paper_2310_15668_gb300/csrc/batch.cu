@@ -13,6 +13,7 @@
 // (no triple crosses two units), so every profile equals what mochy_profile
 // gives for that input and seed.  When the union would not fit the memory
 // budget the inputs are split into waves, each one union and one launch.
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 
@@ -351,19 +352,47 @@ int run_wave(const mochy_config& cfg, const Inputs& in, int g0, int g1, int R, O
 
 // Upper estimate of the device memory one hypergraph needs while it is
 // counted: its line graph has at most sum_v C(d_v, 2) hyperwedges (16 bytes
-// each), plus per-hyperedge, per-incidence and per-node arrays.
-int64_t estimate_graph_bytes(int64_t n_nodes, int64_t n_edges, const int64_t* off,
-                             const int32_t* nodes) {
+// each), plus per-hyperedge, per-incidence and per-node arrays.  On top of it,
+// what the structures that it can do without take: the projection's bitmaps and
+// the levels.  copies: also its randomized copies, whose largest hyperedges are
+// Poisson-like around the input's.
+GraphBytes estimate_graph_bytes(int64_t n_nodes, int64_t n_edges, const int64_t* off,
+                                const int32_t* nodes, int theta, bool copies) {
+  GraphBytes r;
   std::vector<int64_t> deg((size_t)std::max<int64_t>(n_nodes, 0), 0);
   const int64_t T = n_edges > 0 ? off[n_edges] : 0;
   for (int64_t q = 0; q < T; ++q) {
     const int32_t v = nodes[q];
     if (v >= 0 && v < n_nodes) ++deg[(size_t)v];
   }
-  double w = 0.0;
-  for (int64_t d : deg) w += 0.5 * (double)d * (double)(d - 1);
-  return (int64_t)(16.0 * w + 96.0 * (double)n_edges + 48.0 * (double)T +
-                   16.0 * (double)n_nodes) + (1 << 20);
+  double w = 0.0, hubs = 0.0, pairs = 0.0;
+  for (int64_t d : deg) {
+    w += 0.5 * (double)d * (double)(d - 1);
+    hubs += d >= 32 ? 1.0 : 0.0;
+  }
+  int64_t most = 2;
+  for (int64_t e = 0; e < n_edges; ++e) {
+    const int64_t s = std::min<int64_t>(std::max<int64_t>(off[e + 1] - off[e], 0), MOCHY_MAX_EDGE_SIZE);
+    pairs += 0.5 * (double)s * (double)(s - 1);
+    most = std::max(most, s);
+  }
+  if (copies) {
+    const double spread = 6.0 * sqrt((double)most) + 6.0;
+    most = std::min({most + (int64_t)spread, (int64_t)MOCHY_MAX_EDGE_SIZE, std::max<int64_t>(n_nodes, 2)});
+    hubs *= 1.5;
+    pairs *= 1.5;
+  }
+  r.need = (int64_t)(16.0 * w + 96.0 * (double)n_edges + 48.0 * (double)T + 16.0 * (double)n_nodes) +
+           (1 << 20);
+  r.more = (int64_t)(45.0 * (double)T + 10.0 * (double)n_nodes);
+  if (levels_cover(theta, n_edges, 1)) {
+    r.more += (int64_t)levels_bytes((double)n_nodes, (double)n_edges, (double)T, (int)most, theta, w,
+                                    pairs, hubs);
+    // line degrees of 2 w / E on average
+    r.levels = levels_unit_us((double)level_entries((int)most, theta), (double)n_edges) <=
+               split_unit_us((double)n_edges, 4.0 * w * w / (double)n_edges);
+  }
+  return r;
 }
 
 }  // namespace mochy
@@ -394,7 +423,8 @@ extern "C" int mochy_profile_batch(const mochy_config* cfg_in, int32_t n_graphs,
   }
   if (info) memset(info, 0, sizeof(*info));
   // waves: inputs in order, as many per wave as the memory estimate allows
-  // (estimate_graph_bytes per hypergraph and copy); the budget is the
+  // (estimate_graph_bytes per hypergraph and copy, with the levels where these
+  // would count: a wave that has no room for them takes the split kernels); the budget is the
   // configured one, else 70% of the device memory free now.
   int64_t budget = cfg.hbm_budget_bytes;
   if (budget <= 0) {
@@ -406,9 +436,12 @@ extern "C" int mochy_profile_batch(const mochy_config* cfg_in, int32_t n_graphs,
     budget = (int64_t)((double)fr * 0.7);
   }
   std::vector<int64_t> est((size_t)n_graphs);
-  for (int32_t g = 0; g < n_graphs; ++g)
-    est[g] = (int64_t)(n_random + 1) *
-             estimate_graph_bytes(n_nodes[g], n_edges[g], edge_offsets[g], edge_nodes[g]);
+  const bool by_levels = cfg.dense_threshold == 0 && cfg.rest_path == 0;
+  for (int32_t g = 0; g < n_graphs; ++g) {
+    const GraphBytes b = estimate_graph_bytes(n_nodes[g], n_edges[g], edge_offsets[g], edge_nodes[g],
+                                              cfg.theta, true);
+    est[g] = (int64_t)(n_random + 1) * (b.need + (by_levels && b.levels ? b.more : 0));
+  }
   // MOCHY_BATCH_MAX_GRAPHS caps the inputs per wave (smaller unions)
   int32_t cap = n_graphs;
   if (const char* e = getenv("MOCHY_BATCH_MAX_GRAPHS")) {

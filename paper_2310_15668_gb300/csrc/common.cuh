@@ -102,6 +102,9 @@ struct mochy_ctx {
   std::unordered_map<void*, size_t> capacity;   // blocks in use that are larger than asked for
   size_t kept_bytes = 0, kept_max = 0;
   mochy_ctx* copies = nullptr;                  // mochy_profile's randomized copies
+  // bytes that a server reserved for this context (0: no bound): structures that
+  // calls can do without are built within them
+  int64_t reserved = 0;
   int device = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
@@ -238,6 +241,11 @@ int dev_alloc(mochy_ctx* ctx, void** p, size_t bytes);
 void dev_free(mochy_ctx* ctx, void* p, size_t bytes);
 int scratch(mochy_ctx* ctx, int slot, size_t bytes, void** p);
 int drop_scratch(mochy_ctx* ctx, int slot);   // gives one slot's block up
+// is there room, of what is reserved, for a structure that the call can do without?
+inline bool room_for(const mochy_ctx* ctx, size_t bytes) {
+  return ctx->reserved == 0 || ctx->held + (int64_t)bytes <= ctx->reserved;
+}
+size_t scratch_growth(const mochy_ctx* ctx, int slot, size_t bytes);   // bytes that scratch() would add
 void release_scratch(mochy_ctx* ctx);         // all of them
 void release_graph(mochy_ctx* ctx);
 void release_projection(mochy_ctx* ctx);
@@ -276,6 +284,20 @@ int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const 
                   int t1, int t2, PhaseTimer* timer);                 // levels.cu
 void release_levels(mochy_ctx* ctx);                                  // levels.cu
 bool levels_kept(const mochy_ctx* ctx);                               // levels.cu
+double levels_unit_us(double entries, double n_edges);                // levels.cu
+double split_unit_us(double n_edges, double deg2);                    // levels.cu
+int64_t level_entries(int max_size, int theta);                       // levels.cu
+double levels_bytes(double n_nodes, double n_edges, double n_inc, int max_size, int theta,
+                    double wedges, double node_pairs, double hubs);   // levels.cu
+
+// Device memory of one hypergraph while it is counted (batch.cu): what it needs
+// at most, and what the structures that it can do without take at most.
+struct GraphBytes {
+  int64_t need = 0, more = 0;
+  bool levels = false;   // a batch of such hypergraphs would be counted by levels
+};
+GraphBytes estimate_graph_bytes(int64_t n_nodes, int64_t n_edges, const int64_t* off,
+                                const int32_t* nodes, int theta, bool copies);
 int prepare_exact(mochy_ctx* ctx, bool* by_levels);                   // count_split.cu
 int choose_dense_threshold(mochy_ctx* ctx);                           // tune.cu
 int model_split_work(mochy_ctx* ctx, double* sparse, double* words);  // tune.cu

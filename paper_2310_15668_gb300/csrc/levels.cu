@@ -1980,6 +1980,34 @@ bool levels_cover(int theta, int64_t n_edges, int n_units) {
   return theta <= kMaxTheta && n_edges > 0 && n_units < (1 << 18);
 }
 
+double levels_unit_us(double entries, double n_edges) {
+  return 9.3e-5 * pow(entries * n_edges, 0.65);
+}
+
+double split_unit_us(double n_edges, double deg2) {
+  return 0.015 * n_edges + 1.2e-5 * std::min(deg2, 2e4 * n_edges);
+}
+
+int64_t level_entries(int max_size, int theta) {
+  const int Q = theta + 3, S = std::max(max_size, 2);
+  const int64_t n0 = (int64_t)Q * Q * Q;
+  return 2 * n0 + 2 * (S - 1) * n0 + 2 * level2_at(S + 1, Q) + triple_table(theta).total;
+}
+
+// What prepare() takes at most for one hypergraph: heavy pairs share two nodes,
+// so there are no more entries of them than sum_v C(d_v, 2) (wedges).
+double levels_bytes(double n_nodes, double n_edges, double n_inc, int max_size, int theta,
+                    double wedges, double node_pairs, double hubs) {
+  const int Q = theta + 3, CP = Q - 1 <= 4 ? 4 : 8;
+  const double heavy = std::min(wedges, n_edges * n_edges);
+  const double scan = 8.0 * (3.0 * n_edges + 2.0 * n_nodes + 4.0);
+  hubs = std::min(hubs, (double)kMaxHubs);
+  return 2.25 * scan + (4.0 * Q + 44.0) * n_nodes + (12.0 + 4.0 * trip_classes(theta)) * n_edges +
+         2.0 * n_inc + 16.0 * heavy + 16.0 * node_pairs + n_edges * (n_edges + 8.0) / 2.0 +
+         4.0 * (node_pairs + 16.0) * (8.0 + 4.0 * CP) + 4.0 * CP * hubs * hubs +
+         8.0 * (double)level_entries(max_size, theta) + 65536.0;
+}
+
 static unsigned row_grid(const mochy_ctx* ctx, int64_t rows, int per_sm) {
   return (unsigned)std::max<int64_t>(
       1, std::min<int64_t>(ceil_div(rows, kRowWarps), (int64_t)ctx->num_sms * per_sm));
@@ -2059,13 +2087,13 @@ static int levels_pay(mochy_ctx* ctx, int theta, LevelsAgainst against, const Wo
   if (lone || far)   // else in what a unit takes
     levels += 1e-6 * 1024.0 * ((double)w.light_pairs * (7.0 + (far ? 20.0 * f * f : 0.0)) +
                                (double)w.light_rows * (far ? 100.0 : 20.0));
-  levels += lone ? 3.7e-4 * (double)entries : U * 9.3e-5 * pow((double)entries * E / U, 0.65);
+  levels += lone ? 3.7e-4 * (double)entries : U * levels_unit_us((double)entries, E / U);
   if (against == LevelsAgainst::kScan) {
     *pay = levels * (theta + 3) / 4.0 <= 1.25 * (300.0 + 0.03 * E + 1e-5 * deg2);
     return MOCHY_OK;
   }
   *pay = levels <= (lone ? 1.3 * (340.0 + 0.01 * E + 5e-6 * deg2)
-                         : 340.0 + 0.015 * E + 1.2e-5 * std::min(deg2, 2e4 * E));
+                         : 340.0 + split_unit_us(E, deg2));
   if (*pay || !lone) return MOCHY_OK;
   double sparse = 0.0, words = 0.0;
   const int rc = model_split_work(ctx, &sparse, &words);
@@ -2113,6 +2141,8 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against)
                b_unit = al((size_t)U * sizeof(LevelUnit)),
                b_tot = al((size_t)(3 + 2 * (U + 1) + 3) * 8);
   lv->bytes[0] = b_scan + b_ncls + 2 * b_hplus + b_ehub + b_unit + b_tot;
+  if (!room_for(ctx, lv->bytes[0] + scratch_growth(ctx, 0, (size_t)(n_seg + 1) * 8 + sizeof(Work))))
+    return fail(MOCHY_E_NOMEM, "level structures past the reserved memory");
   MOCHY_TRY(dev_alloc(ctx, &lv->block[0], lv->bytes[0]));
   char* c = (char*)lv->block[0];
   auto carve = [&](size_t b) { char* r = c; c += b; return r; };
@@ -2223,6 +2253,8 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against)
                b_hubm = al((size_t)std::max<int64_t>(hub_pairs, 1) * g.CP * 4),
                b_tab = al((size_t)U * g.tab_stride * 8), b_other = al(oslots * 16);
   lv->bytes[1] = b_hadj + b_adj + b_list + b_first + b_mat + b_key + b_cnt + b_cur + b_hubm + b_tab + b_other + 256;
+  if (!room_for(ctx, lv->bytes[1]))
+    return fail(MOCHY_E_NOMEM, "level structures past the reserved memory");
   MOCHY_TRY(dev_alloc(ctx, &lv->block[1], lv->bytes[1]));
   c = (char*)lv->block[1];
   uint2* hadj = (uint2*)carve(b_hadj);

@@ -328,7 +328,8 @@ int project_graph(mochy_ctx* ctx) {
   // line graph needs.
   const size_t b_nodes = (size_t)ctx->n_nodes * 8, b_bits = (size_t)ctx->n_inc * 36 + 256;
   void* t2 = nullptr;
-  const int rc2 = scratch(ctx, 2, b_nodes + 8 + b_bits, &t2);
+  const int rc2 = room_for(ctx, scratch_growth(ctx, 2, b_nodes + 8 + b_bits))
+                      ? scratch(ctx, 2, b_nodes + 8 + b_bits, &t2) : MOCHY_E_NOMEM;
   if (rc2 < 0 && rc2 != MOCHY_E_NOMEM) return rc2;
   if (rc2 < 0) t2 = nullptr;
   ProjArgs g;

@@ -839,7 +839,10 @@ int count_sampled(mochy_ctx* ctx, int method, int64_t samples, uint64_t seed,
     if (method == MOCHY_A_PLUS) {
       // the draws, grouped by row when there are enough for rows to repeat
       const bool group = samples >= kGroupDraws;
-      rc = scratch(ctx, 0, (size_t)samples * 16 + 16, &t);
+      // (with the sort's scratch, 24 bytes a draw and a few KB)
+      rc = room_for(ctx, scratch_growth(ctx, 0, (size_t)samples * 16 + 16) +
+                             (group ? scratch_growth(ctx, 1, (size_t)samples * 24 + (1 << 16)) : 0))
+               ? scratch(ctx, 0, (size_t)samples * 16 + 16, &t) : MOCHY_E_NOMEM;
       if (rc == MOCHY_OK) {
         uint2* other = (uint2*)t;
         uint32_t* row = (uint32_t*)(other + samples);
@@ -853,7 +856,8 @@ int count_sampled(mochy_ctx* ctx, int method, int64_t samples, uint64_t seed,
       }
     } else {
       r.n_classes = std::max(ctx->max_size, 1) * (ctx->theta + 2);
-      rc = scratch(ctx, 2, (size_t)r.n_classes * ctx->n_edges * 4, &t);
+      rc = room_for(ctx, scratch_growth(ctx, 2, (size_t)r.n_classes * ctx->n_edges * 4))
+               ? scratch(ctx, 2, (size_t)r.n_classes * ctx->n_edges * 4, &t) : MOCHY_E_NOMEM;
       if (rc == MOCHY_OK) {
         k_row_classes<<<(unsigned)std::min<int64_t>(ceil_div(ctx->n_edges, kRowsWarps),
                                                     (int64_t)ctx->num_sms * 8),

@@ -3,7 +3,9 @@
 // count, sampled count or characteristic profile of a hypergraph) wait in a
 // queue and are admitted, in arrival order, as soon as a slot is free and
 // their estimated device memory fits the budget beside the requests already
-// running.  Requests that arrive while others run are admitted as slots and
+// running; what is left then is reserved for structures that they can do
+// without (the levels of an exact count, bitmaps, class histograms), which are
+// only built within the reservation.  Requests that arrive while others run are admitted as slots and
 // memory free up, and their work overlaps on the device through the slots'
 // streams.  Every request runs the same library calls as a direct caller
 // would (mochy_load, mochy_project, then mochy_count_exact,
@@ -26,8 +28,6 @@
 
 namespace mochy {
 
-int64_t estimate_graph_bytes(int64_t n_nodes, int64_t n_edges, const int64_t* off,
-                             const int32_t* nodes);   // batch.cu
 void keep_no_blocks(mochy_ctx* ctx);                  // api.cu
 
 namespace {
@@ -45,7 +45,9 @@ struct Request {
   int64_t samples = 0;
   int32_t n_random = 0;
   uint64_t seed = 0;
-  int64_t est = 0;
+  int64_t est = 0;           // bytes it needs
+  int64_t more = 0;          // bytes of structures that it can do without
+  int64_t granted = 0;       // bytes reserved while it runs
   int32_t bypassed = 0;      // later requests admitted while this one waited
   bool onthefly = false;     // MoCHy-A+ without the line graph
   int64_t otf_budget = 0;    // its bitmap budget, bytes
@@ -93,6 +95,8 @@ namespace mochy {
 namespace {
 
 void run_request(mochy_ctx* ctx, const Request& r, mochy_result& out) {
+  // a profile's context and that of its copies take half each
+  ctx->reserved = r.kind == MOCHY_REQ_PROFILE ? r.granted / 2 : r.granted;
   int rc = mochy_load(ctx, r.n_nodes, (int64_t)r.off.size() - 1, r.off.data(),
                       r.nodes.empty() ? nullptr : r.nodes.data(), nullptr);
   if (rc >= 0 && r.onthefly) {
@@ -171,7 +175,12 @@ void worker_main(mochy_server* s) {
       if (it != s->pending.begin()) s->pending.front()->bypassed += 1;
       r = std::move(*it);
       s->pending.erase(it);
-      s->reserved += r->est;
+      // what it can do without is granted from what the oldest waiting request
+      // leaves over
+      int64_t left = s->budget - s->reserved - r->est;
+      if (!s->pending.empty()) left -= s->pending.front()->est;
+      r->granted = r->est + std::min(r->more, std::max<int64_t>(left, 0));
+      s->reserved += r->granted;
       s->peak_reserved = std::max(s->peak_reserved, s->reserved);
       s->in_flight += 1;
       s->peak_in_flight = std::max(s->peak_in_flight, s->in_flight);
@@ -186,7 +195,7 @@ void worker_main(mochy_server* s) {
     res->latency_ms = t_end - r->t_submit;
     {
       std::lock_guard<std::mutex> lk(s->mu);
-      s->reserved -= r->est;
+      s->reserved -= r->granted;
       s->in_flight -= 1;
       if (res->status >= 0) {
         s->completed += 1;
@@ -266,14 +275,22 @@ int mochy_server_submit(mochy_server* s, const mochy_request* req, int64_t* tick
   r->n_random = req->n_random;
   r->seed = req->seed;
   // a profile holds the input and one copy at a time
-  r->est = estimate_graph_bytes(req->n_nodes, req->n_edges, req->edge_offsets, req->edge_nodes) *
-           (req->kind == MOCHY_REQ_PROFILE ? 2 : 1);
+  const GraphBytes b = estimate_graph_bytes(req->n_nodes, req->n_edges, req->edge_offsets,
+                                            req->edge_nodes, s->cfg.theta,
+                                            req->kind == MOCHY_REQ_PROFILE);
+  r->est = b.need * (req->kind == MOCHY_REQ_PROFILE ? 2 : 1);
+  r->more = b.more * (req->kind == MOCHY_REQ_PROFILE ? 2 : 1);
+  if (req->kind == MOCHY_REQ_SAMPLED)   // the projection's bitmaps, class histograms, draws
+    r->more = (int64_t)(45.0 * (double)T + 10.0 * (double)req->n_nodes +
+                        5.0 * MOCHY_MAX_EDGE_SIZE * (s->cfg.theta + 2) * (double)req->n_edges +
+                        50.0 * (double)req->samples) + (1 << 17);
   // a MoCHy-A+ request whose line graph would take more than a quarter of
   // the budget runs without it (identical results; the memory is the
   // hypergraph, the degree arrays and the membership bitmaps)
   if (req->kind == MOCHY_REQ_SAMPLED && req->method == MOCHY_A_PLUS && r->est > s->budget / 4) {
     r->onthefly = true;
     r->otf_budget = std::min<int64_t>(s->budget / 8, (int64_t)1 << 30);
+    r->more = 0;
     r->est = (int64_t)(64.0 * (double)req->n_edges + 48.0 * (double)T +
                        20.0 * (double)req->n_nodes) + r->otf_budget + ((int64_t)1 << 20);
   }

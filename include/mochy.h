@@ -67,13 +67,15 @@ typedef struct {
   void* stream;             /* cudaStream_t to run on; NULL = own stream */
   int32_t exact_kernel;     /* mochy_count_exact: 0 = open pairs counted per
                                centre, closed ones by levels of overlap (theta
-                               up to 4), else by the split kernels (closed ones
+                               up to 4) where that takes less time and fits,
+                               else by the split kernels (closed ones
                                enumerated; see dense_threshold), 1 = plain
                                per-hyperwedge scan; all give the same counts */
   int32_t dense_threshold;  /* split kernels: line degree from which a row is
                                kept as a bitmap; 0 = chosen by the tuner.  A
-                               positive value, or a rest_path, makes exact
-                               counts take the split kernels */
+                               positive value, a rest_path, or a call of
+                               mochy_tune_dense_threshold makes exact counts
+                               take the split kernels */
   int32_t rest_path;        /* split kernel, closed candidates of dense rows
                                outside the popcounted combinations: 1 = each
                                lane classifies those of its own word, 2 = they
@@ -173,7 +175,8 @@ int mochy_count_exact_rows(mochy_ctx* ctx, const int32_t* h_rows, int64_t n_rows
  * built and the split count of one seeded sample of rows (each row kept
  * with probability sample_fraction by a SplitMix64 hash of (seed, row)) is
  * timed with CUDA events on the context's stream.  The fastest threshold
- * becomes the context's dense threshold for the following counts and is
+ * becomes the context's dense threshold for the following counts, which take
+ * the split kernels from then on (as with a configured one), and is
  * written to *best (may be NULL); tried and ms (may be NULL; n_candidates
  * entries, 5 for the default list) receive each candidate and its time in
  * milliseconds, -1 where its structures did not fit (device memory or the
@@ -231,9 +234,9 @@ int mochy_radial_node_profile(mochy_ctx* ctx, int64_t* np_h, int64_t* np_3h);
  * out_kh[t-1] (cap >= X(k) entries, may be NULL) receives the count of
  * kh-motif t, out_h (26, may be NULL) the h-motif counts, *n_motifs (may be
  * NULL) X(k).  Thresholds up to 4 are counted by levels of overlap like
- * mochy_count_exact; with larger ones, or where those arrays do not fit,
- * instances are enumerated one by one by the per-hyperwedge scan
- * (exact_kernel = 1's kernel).  At most about 300,000 hyperedges either way.
+ * mochy_count_exact where that takes less time; with larger ones, or where
+ * those arrays do not fit, instances are enumerated one by one by the
+ * per-hyperwedge scan (exact_kernel = 1's kernel).  At most about 300,000 hyperedges either way.
  * Needs mochy_project. */
 int mochy_count_kh(mochy_ctx* ctx, int32_t k, const int32_t* thresholds, int64_t* out_h,
                    int64_t* out_kh, int64_t cap, int64_t* n_motifs);
@@ -332,7 +335,8 @@ int mochy_profile(mochy_ctx* ctx, int32_t n_random, uint64_t seed,
 typedef struct {
   double ms_generate;   /* inputs loaded, copies drawn, transformed and loaded */
   double ms_project;    /* line graph of the union */
-  double ms_prepare;    /* split structures (dense index, bitmaps) */
+  double ms_prepare;    /* level structures (tables, overlap matrix) or split
+                           structures (dense index, bitmaps) */
   double ms_count;      /* the one CUDA-graph launch of the counting kernels */
   double ms_finish;     /* per-hypergraph counts, significance, CP, copy-out */
   int64_t n_waves;      /* unions counted (1 unless memory forced a split) */
@@ -341,7 +345,7 @@ typedef struct {
   int64_t n_edges;      /* hyperedges of the unions (after duplicate removal) */
   int64_t n_wedges;     /* hyperwedges of the unions */
   int64_t instances;    /* connected triples counted, all hypergraphs */
-  int32_t dense_threshold;
+  int32_t dense_threshold;  /* of the last wave's split kernels; 0: by levels */
 } mochy_batch_info;
 
 /* Significance and characteristic profiles (Eq. "significance", Eq. "cp",

@@ -972,7 +972,7 @@ int mochy_trace_read(mochy_ctx* ctx, char* buf, int64_t len) {
            "\"heavy_bitmaps\": %llu, \"slots_evicted\": %llu, \"slots_flushed_full\": %llu, "
            "\"dense_rows_counted\": %llu, \"otf_candidates\": %llu, \"otf_words\": %llu, "
            "\"otf_list_entries\": %llu, \"otf_exact\": %llu, \"otf_bitmaps\": %lld}",
-           (long long)ctx->n_dense, ctx->split_ready ? ctx->dense_thr_used : ctx->dense_thr,
+           (long long)ctx->n_dense, ctx->trace_thr,
            (long long)ctx->wwords,
            (long long)ctx->n_heavy, st[0], st[1], st[2], st[3], st[4], st[5], st[6], st[7], st[8],
            st[9], st[10], st[11], st[12], st[13], st[14], st[16], st[17], st[18], st[19],

@@ -182,7 +182,8 @@ struct mochy_ctx {
   double model_sparse = 0.0, model_words = 0.0;   // what it leaves the split kernels to do
   cudaStream_t side[mochy::kSides] = {};        // its independent kernels run side by side
   cudaEvent_t side_ev[mochy::kSides + 1] = {};
-  bool split_forced = false;     // the configuration asks for the split kernels
+  bool split_forced = false;     // the configuration or the measured tuner asks for the split kernels
+  int trace_thr = 0;             // dense threshold of the last exact count, 0: it had none
 
   // MoCHy-A+ without the line graph (built on first use after a load):
   // membership bitmaps of the most popular nodes, size planes, and the

@@ -1717,8 +1717,9 @@ static int launch_split(mochy_ctx* ctx, SplitPlan p, PhaseTimer* timer, const Wo
 }
 
 // Builds what the exact count of this context needs and says which kernels
-// it takes: by levels of overlap (levels.cu), unless the configuration asks
-// for the split kernels (dense_threshold or rest_path), theta is past what the
+// it takes: by levels of overlap (levels.cu), unless the configuration
+// (dense_threshold or rest_path) or the measured tuner asks for the split
+// kernels, theta is past what the
 // level tables hold, the split kernels take less time (levels_pay in
 // levels.cu), or the level structures do not fit the device memory.
 int prepare_exact(mochy_ctx* ctx, bool* by_levels) {
@@ -1754,6 +1755,7 @@ int count_exact_split(mochy_ctx* ctx, unsigned long long* d_hist) {
     if (by_levels) {
       MOCHY_TRY(launch_levels(ctx, d_hist, 432, ctx->tables.lut3, 3, ctx->theta, 1 << 30, &timer));
       timer.report(ctx);
+      ctx->trace_thr = 0;
       return MOCHY_OK;
     }
     timer.restart();
@@ -1776,6 +1778,7 @@ int count_exact_split(mochy_ctx* ctx, unsigned long long* d_hist) {
     MOCHY_TRY(launch_split<false>(ctx, plan, &timer, all_rows(ctx)));
   }
   timer.report(ctx);
+  ctx->trace_thr = ctx->dense_thr_used;
   return MOCHY_OK;
 }
 
@@ -1839,6 +1842,7 @@ int count_split_rows(mochy_ctx* ctx, const int32_t* d_rows, int64_t n_rows,
   wl.n_dense = (int64_t)hc[1];
   MOCHY_TRY(launch_split<false>(ctx, plan, &timer, wl));
   timer.report(ctx);
+  ctx->trace_thr = ctx->dense_thr_used;
   return MOCHY_OK;
 }
 

@@ -185,7 +185,15 @@ int tune_dense_threshold(mochy_ctx* ctx, const int32_t* cand, int32_t n_cand, do
     ctx->dense_thr = saved;
     return fail(MOCHY_E_UNSUPPORTED, "no candidate threshold fits");
   }
+  // the following counts are the split kernels', with this threshold, as with a
+  // configured one; the copies' context of mochy_profile is made anew with it
   ctx->dense_thr = best;
+  ctx->split_forced = true;
+  release_levels(ctx);
+  if (ctx->copies) {
+    mochy_destroy(ctx->copies);
+    ctx->copies = nullptr;
+  }
   if (best_out) *best_out = best;
   return MOCHY_OK;
 }

@@ -472,7 +472,11 @@ int mochy_trace_read(mochy_ctx* ctx, char* buf, int64_t len);
 /* Bytes of device memory the context holds now.  Not counted are the blocks
  * that it has given up and keeps for its next allocations: at most 16 GB and
  * 64 blocks, within hbm_budget_bytes where one is set, given back when an
- * allocation of any context on the device would fail, and by mochy_destroy. */
+ * allocation of any context on the device would fail, and by mochy_destroy.
+ * Nothing else gives them back to another allocator of the process; the default
+ * budgets of batches and servers count them as free.  Nor is the context that
+ * mochy_profile keeps for its copies when there is no budget (motif tables and a
+ * stream; its kept blocks are within the same bounds). */
 int64_t mochy_device_bytes(mochy_ctx* ctx);
 
 /* Number of kernels the library launched in this process (for accounting). */

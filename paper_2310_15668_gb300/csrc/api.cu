@@ -57,11 +57,12 @@ int ensure_dynamic_smem(const void* func, size_t bytes) {
 // the same context, so in the order of its stream; the side streams are joined
 // before anything is given up.  It serves requests of its size down to four
 // fifths of it (and 64 KB less), or, under a budget, of its size alone.
-//   Bounds: kKeptBytes and kKeptBlocks a context, oldest first; a context with
-// a budget keeps no more than the budget leaves; an allocation that fails gives
-// back what every context on the device keeps and tries again; mochy_destroy
-// gives back the rest.  A server's contexts keep none: their memory is
-// reserved by request.
+//   Bounds: kKeptBytes and kKeptBlocks a context and its copies' context
+// together, the idle one's first, oldest first; a context with a budget keeps no
+// more than the budget leaves; an allocation that fails gives back what every
+// context on the device keeps and tries again, so what is kept counts as free
+// where a default budget is made from the free memory; mochy_destroy gives back
+// the rest.  A server's contexts keep none: their memory is reserved by request.
 namespace {
 
 constexpr size_t kKeptBytes = (size_t)16 << 30;   // an eighteenth of the device's memory
@@ -74,6 +75,12 @@ void give_back(mochy_ctx* ctx) {
   for (auto& k : ctx->kept) cudaFree(k.p);
   ctx->kept.clear();
   ctx->kept_bytes = 0;
+}
+
+void give_back_oldest(mochy_ctx* ctx) {
+  cudaFree(ctx->kept.front().p);
+  ctx->kept_bytes -= ctx->kept.front().bytes;
+  ctx->kept.erase(ctx->kept.begin());
 }
 
 }  // namespace
@@ -90,8 +97,24 @@ void keep_no_blocks(mochy_ctx* ctx) {
   std::lock_guard<std::mutex> lk(kept_mu);
   ctx->kept_max = 0;
   give_back(ctx);
+  if (ctx->kept_with) ctx->kept_with->kept_with = nullptr;
+  ctx->kept_with = nullptr;
   kept_contexts.erase(std::remove(kept_contexts.begin(), kept_contexts.end(), ctx),
                       kept_contexts.end());
+}
+
+void keep_together(mochy_ctx* ctx, mochy_ctx* copies) {
+  std::lock_guard<std::mutex> lk(kept_mu);
+  ctx->kept_with = copies;
+  copies->kept_with = ctx;
+}
+
+size_t kept_on_device(int device) {
+  std::lock_guard<std::mutex> lk(kept_mu);
+  size_t bytes = 0;
+  for (const mochy_ctx* c : kept_contexts)
+    if (c->device == device) bytes += c->kept_bytes;
+  return bytes;
 }
 
 // An allocation that the budget or the device refuses is tried once more without
@@ -168,11 +191,10 @@ void dev_free(mochy_ctx* ctx, void* p, size_t bytes) {
   }
   ctx->kept.push_back({p, bytes});
   ctx->kept_bytes += bytes;
-  while (ctx->kept_bytes > ctx->kept_max || ctx->kept.size() > kKeptBlocks) {
-    cudaFree(ctx->kept.front().p);
-    ctx->kept_bytes -= ctx->kept.front().bytes;
-    ctx->kept.erase(ctx->kept.begin());
-  }
+  mochy_ctx* idle = ctx->kept_with;
+  while (ctx->kept_bytes + (idle ? idle->kept_bytes : 0) > ctx->kept_max ||
+         ctx->kept.size() + (idle ? idle->kept.size() : 0) > kKeptBlocks)
+    give_back_oldest(idle && !idle->kept.empty() ? idle : ctx);
 }
 
 int drop_scratch(mochy_ctx* ctx, int slot) {
@@ -891,6 +913,7 @@ int mochy_profile(mochy_ctx* ctx, int32_t n_random, uint64_t seed, double* sig_h
   ctx->copies = nullptr;
   if (rc == MOCHY_OK && !copy_ctx) rc = new_like(ctx, &copy_ctx);
   if (rc == MOCHY_OK && ctx->kept_max == 0) keep_no_blocks(copy_ctx);
+  if (rc == MOCHY_OK && ctx->kept_max > 0) keep_together(ctx, copy_ctx);
   if (rc == MOCHY_OK) copy_ctx->reserved = ctx->reserved;
   for (int32_t c = 0; rc == MOCHY_OK && c < n_random; ++c) {
     rc = randomize_graph(ctx, seed, (uint32_t)c, copy_ctx);

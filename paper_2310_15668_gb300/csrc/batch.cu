@@ -433,7 +433,7 @@ extern "C" int mochy_profile_batch(const mochy_config* cfg_in, int32_t n_graphs,
       cudaGetLastError();
       return fail(MOCHY_E_CUDA, "cannot query device memory");
     }
-    budget = (int64_t)((double)fr * 0.7);
+    budget = (int64_t)((double)(fr + kept_on_device(cfg.device)) * 0.7);
   }
   std::vector<int64_t> est((size_t)n_graphs);
   const bool by_levels = cfg.dense_threshold == 0 && cfg.rest_path == 0;

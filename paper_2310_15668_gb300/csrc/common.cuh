@@ -101,6 +101,7 @@ struct mochy_ctx {
   std::vector<Kept> kept;
   std::unordered_map<void*, size_t> capacity;   // blocks in use that are larger than asked for
   size_t kept_bytes = 0, kept_max = 0;
+  mochy_ctx* kept_with = nullptr;               // shares the bounds: its copies' context, or theirs
   mochy_ctx* copies = nullptr;                  // mochy_profile's randomized copies
   // bytes that a server reserved for this context (0: no bound): structures that
   // calls can do without are built within them
@@ -246,6 +247,7 @@ int drop_scratch(mochy_ctx* ctx, int slot);   // gives one slot's block up
 inline bool room_for(const mochy_ctx* ctx, size_t bytes) {
   return ctx->reserved == 0 || ctx->held + (int64_t)bytes <= ctx->reserved;
 }
+size_t kept_on_device(int device);            // bytes that all contexts keep, given back on demand
 size_t scratch_growth(const mochy_ctx* ctx, int slot, size_t bytes);   // bytes that scratch() would add
 void release_scratch(mochy_ctx* ctx);         // all of them
 void release_graph(mochy_ctx* ctx);

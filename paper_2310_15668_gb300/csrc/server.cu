@@ -238,7 +238,7 @@ int mochy_server_create(mochy_server** out, const mochy_config* cfg, int32_t n_s
       delete s;
       return fail(MOCHY_E_CUDA, "cannot query device memory");
     }
-    s->budget = (int64_t)((double)fr * 0.7);
+    s->budget = (int64_t)((double)(fr + kept_on_device(s->cfg.device)) * 0.7);
   }
   for (int32_t i = 0; i < n_slots; ++i) s->workers.emplace_back(worker_main, s);
   *out = s;

@@ -199,3 +199,52 @@ def test_kh_motifs_of_a_sparse_hypergraph(theta):
         h, h3 = c.count_exact()
         kh, k3 = c.count_kh(3, (theta,))
     assert np.array_equal(h, kh) and np.array_equal(h3, k3)
+
+
+def _groups(shared, own, counts):
+    """For each count a group of that many hyperedges with `shared` nodes in
+    common and `own` of their own: count - 1 heavy pairs each; and hyperedges
+    across the groups, of one node of each."""
+    sets, n, firsts = [], 0, []
+    for k in counts:
+        base = tuple(range(n, n + shared))
+        firsts.append(n)
+        n += shared
+        for _ in range(k):
+            sets.append(base + tuple(range(n, n + own)))
+            n += own
+    sets += [tuple(firsts), tuple(f + shared for f in firsts), (firsts[0], firsts[-1])]
+    return (n, *_util.csr_from_sets(sets))
+
+
+def _heavy_degrees(g):
+    n, off, nodes = g
+    m = np.zeros((len(off) - 1, n), np.int32)
+    for i in range(len(off) - 1):
+        m[i, nodes[off[i]:off[i + 1]]] = 1
+    om = m @ m.T
+    np.fill_diagonal(om, 0)
+    return (om >= 2).sum(1)
+
+
+@pytest.mark.parametrize("theta", [1, 4])
+@pytest.mark.parametrize("shared,own", [(2, 1), (3, 2), (30, 4)])
+def test_rows_of_16_and_17_heavy_pairs(shared, own, theta):
+    """Rows of up to 16 heavy pairs are counted pair by pair, longer ones by
+    classes; hyperedges of more than 32 nodes have no node masks."""
+    g = _groups(shared, own, (16, 17, 18, 33, 34))
+    assert {15, 16, 17, 32, 33} <= set(_heavy_degrees(g).tolist())
+    h, h3 = _count(g, theta=theta)
+    oh, o3 = oracle.count_exact(g[1], g[2], theta=theta)
+    assert np.array_equal(h, oh) and np.array_equal(h3, o3)
+
+
+def test_rows_of_16_and_17_heavy_pairs_in_a_batch():
+    gs = [_groups(s, o, c) for s, o, c in ((2, 1, (17, 18)), (3, 2, (16, 17, 18)), (30, 4, (18, 17)))]
+    gs = [g for g in gs for _ in range(3)]
+    seeds = list(range(len(gs)))
+    _, _, _, _, ch, c3, _, info = B.mochy_profile_batch(gs, 1, seeds)
+    assert info["dense_threshold"] == 0      # by levels
+    for g, (n, off, nodes) in enumerate(gs):
+        o = oracle.profile(n, off, nodes, 1, seeds[g])
+        assert np.array_equal(ch[g], o["counts_h"]) and np.array_equal(c3[g], o["counts_3h"])

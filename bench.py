@@ -419,12 +419,13 @@ def _tuner_measure(ctx, st):
     """The measured dense-threshold tuner on the bench hypergraph, after the
     timed steps: each of its candidate thresholds times the dense count of
     the same 2 % row sample with CUDA events, and the fastest is its pick;
-    reported beside the threshold the timed steps used."""
+    reported beside the threshold of the step at trace level 2 (the timed steps
+    count by levels, which have none)."""
     from paper_2310_15668_gb300 import binding as B
     t = time.perf_counter()
     best, tried = B.mochy_tune_dense_threshold(ctx.h)
     return {"kind": "measured (CUDA events on a 2 % row sample per candidate)",
-            "threshold_of_timed_steps": int(st.get("dense_threshold", 0)), "best": int(best),
+            "threshold_of_traced_step": int(st.get("dense_threshold", 0)), "best": int(best),
             "candidates_ms": {str(int(thr)): float(ms) for thr, ms in tried},
             "seconds": time.perf_counter() - t}
 

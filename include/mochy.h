@@ -357,8 +357,8 @@ typedef struct {
  * inputs and their randomized copies are generated on the device, as one
  * disjoint union per wave (as many inputs as the configured memory budget,
  * else 70% of the free device memory, allows), and every hypergraph of the
- * union is counted exactly by one launch of a CUDA graph of persistent
- * work-queue kernels.  Outputs (host, caller-allocated, each may be NULL):
+ * union is counted exactly by one launch of a CUDA graph of the counting
+ * kernels.  Outputs (host, caller-allocated, each may be NULL):
  * sig_h, cp_h [n_graphs][26]; sig_3h, cp_3h [n_graphs][431]; counts_h
  * [n_graphs][1 + n_random][26] and counts_3h [n_graphs][1 + n_random][431]
  * (the input first, then copies 0..); degenerate [n_graphs] (1 when all

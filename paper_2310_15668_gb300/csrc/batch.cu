@@ -5,11 +5,11 @@
 //
 // The inputs and all their copies form one disjoint union of "units" (unit
 // g (R+1) is input g, unit g (R+1) + 1 + c its copy c), each with its own node
-// and hyperedge ranges.  The union is projected once; the split exact count
-// (count_split.cu) keeps a dense index space, bitmap windows and a histogram
-// per unit, and its three persistent work-queue kernels run over the rows of
-// every unit at once, captured into one CUDA graph and replayed by a single
-// launch.  A unit's counts are exactly those of its hypergraph counted alone
+// and hyperedge ranges.  The union is projected once; the exact count keeps
+// tables, overlap matrix and histogram (by levels, levels.cu) or a dense index
+// space, bitmap windows and histogram (split kernels, count_split.cu) per unit,
+// and its kernels run over the rows of every unit at once, captured into one
+// CUDA graph and replayed by a single launch.  A unit's counts are exactly those of its hypergraph counted alone
 // (no triple crosses two units), so every profile equals what mochy_profile
 // gives for that input and seed.  When the union would not fit the memory
 // budget the inputs are split into waves, each one union and one launch.
@@ -271,7 +271,7 @@ int run_wave(const mochy_config& cfg, const Inputs& in, int g0, int g1, int R, O
   }
   MOCHY_TRY(set_units(cx, nseg));
   cudaEventRecord(ev.e[1], cx->stream);
-  // 4. the union's line graph and split structures
+  // 4. the union's line graph and level or split structures
   MOCHY_TRY(project_graph(cx));
   cudaEventRecord(ev.e[2], cx->stream);
   bool by_levels;

@@ -330,6 +330,14 @@ int significance_cp_batch(mochy_ctx* ctx, const int64_t* d_counts_h, const int64
                           int n_graphs, int32_t n_random, double eps, double* d_out,
                           int32_t* d_degenerate);                     // profile.cu
 
+// 64-bit finaliser of MurmurHash3 (Appleby, public domain; the constants are
+// its own), for open-addressing tables
+__device__ __forceinline__ uint64_t mix64(uint64_t z) {
+  z ^= z >> 33; z *= 0xff51afd7ed558ccdull;
+  z ^= z >> 33; z *= 0xc4ceb9fe1a85ec53ull;
+  return z ^ (z >> 33);
+}
+
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 // largest u in [0, n) with b[u] <= x, for ascending b with b[0] <= x (with

@@ -146,12 +146,6 @@ __device__ __forceinline__ int unit_of(const int64_t* seg, int n, int64_t i) {
   return n > 1 ? seg_of(seg, n, i) : 0;
 }
 
-__device__ __forceinline__ uint64_t mix(uint64_t z) {
-  z ^= z >> 33; z *= 0xff51afd7ed558ccdull;
-  z ^= z >> 33; z *= 0xc4ceb9fe1a85ec53ull;
-  return z ^ (z >> 33);
-}
-
 // a pair {a, b}: is b after a in the order (heavy degree, id)?
 __device__ __forceinline__ bool after(int64_t hb, int64_t b, int64_t ha, int64_t a) {
   return hb != ha ? hb > ha : b > a;
@@ -185,7 +179,7 @@ __device__ __forceinline__ bool in_sorted(const int32_t* s, int n, int32_t u) {
 // slot of node pair u < w, or -1
 __device__ __forceinline__ int64_t find_pair(const LevelArgs& g, int32_t u, int32_t w) {
   const uint64_t key = ((uint64_t)(uint32_t)min(u, w) << 32) | (uint32_t)max(u, w);
-  uint64_t s = mix(key) & g.hmask;
+  uint64_t s = mix64(key) & g.hmask;
   for (uint64_t probe = 0; probe <= g.hmask; ++probe) {
     const uint64_t k = __ldg(&g.hkey[s]);
     if (k == key) return (int64_t)s;
@@ -481,7 +475,7 @@ k_lv_pairs(LevelArgs g, const int64_t* __restrict__ bscan, uint64_t* __restrict_
       while ((j + 1) * j / 2 <= n) ++j;
       const int i = n - j * (j - 1) / 2;
       const uint64_t key = ((uint64_t)(uint32_t)nodes[warp][i] << 32) | (uint32_t)nodes[warp][j];
-      uint64_t s = mix(key) & g.hmask;
+      uint64_t s = mix64(key) & g.hmask;
       for (uint64_t probe = 0; probe <= g.hmask; ++probe) {
         unsigned long long k = hkey[s];
         if (k == 0ull) k = atomicCAS((unsigned long long*)&hkey[s], 0ull, (unsigned long long)key);
@@ -1349,7 +1343,7 @@ __device__ __noinline__ void trip_other(const LevelArgs& g, const Coder& cd,
   const unsigned long long key =
       1ull + ((((((((unsigned long long)unit << 6 | t) << 6 | p) << 6 | q) << 6 | r) << 7 | a1) << 7 |
                b1) << 7 | c1);
-  uint64_t s = mix(key) & g.omask;
+  uint64_t s = mix64(key) & g.omask;
   for (int probe = 0; probe < 256; ++probe) {
     unsigned long long k = g.okey[s];
     if (k == 0ull) k = atomicCAS(&g.okey[s], 0ull, key);

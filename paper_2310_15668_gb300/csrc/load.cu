@@ -31,12 +31,6 @@ __global__ void k_validate_sort(const int64_t* __restrict__ off, const int32_t* 
   for (int q = 0; q < (int)s; ++q) sorted[b + q] = v[q];
 }
 
-__device__ __forceinline__ uint64_t mix64(uint64_t z) {
-  z ^= z >> 33; z *= 0xff51afd7ed558ccdull;
-  z ^= z >> 33; z *= 0xc4ceb9fe1a85ec53ull;
-  return z ^ (z >> 33);
-}
-
 __device__ uint64_t edge_hash(const int32_t* nodes, int64_t b, int64_t e) {
   uint64_t h = 0x9e3779b97f4a7c15ull ^ (uint64_t)(e - b);
   for (int64_t q = b; q < e; ++q) h = mix64(h ^ (uint64_t)(uint32_t)nodes[q]) + 0x632be59bd9b4e019ull;

@@ -9,9 +9,9 @@
 //        Algorithm sampling_ver1).
 // Two kernels do this.  k_sample_merge: a warp merges the sorted rows of e_i
 // and e_j tile by tile (short rows, or more hyperedges than shared memory has
-// codes for).  k_sample_rows: a block keeps the overlaps of row e_i as 2-bit
-// codes in shared memory and only streams row e_j; what e_i is the centre of
-// comes from a histogram of its row.
+// codes for).  k_sample_pairs (A+) and k_sample_rows (A): a block keeps the
+// overlaps of one row as 4-bit codes in shared memory and only streams the
+// other; what the first is the centre of comes from a histogram of its row.
 // Random draws: Philox4x32-10 (Salmon et al., SC'11) on counter
 // (n_lo, n_hi, stream, 0) with key (seed_lo, seed_hi); the 64-bit output u
 // selects floor(u * range / 2^64).
@@ -171,21 +171,21 @@ k_sample_merge(SampleArgs g, int64_t n_items) {
 
 // ---------------------------------------------------------------------------
 // Work items of long rows.  For a hyperwedge of a staged row e_i and a streamed
-// row e_j, with the staged row as codes min(omega, 3) and as a histogram of
+// row e_j, with the staged row as codes min(omega, 14) and as a histogram of
 // classes (omega_ik, min(|e_k| - omega_ik, theta + 1)),
 //   * e_k in N_j \ N_i (open, centre e_j) and e_k in N_i & N_j (closed) are
 //     found by streaming row e_j alone;
 //   * the open instances with centre e_i are the pairs (e_j, e_k) of the
 //     histogram, less one "as if open" term for every closed instance.
 // A+ stages the longer of its two rows and groups the draws by it.  A, which
-// takes closed instances with j < k only, streams just those entries when it
-// has many samples: the pairs of every centre e_j then come from class
+// takes closed instances with j < k only, streams just those entries: the
+// pairs of every centre e_j come from class
 // histograms of all rows, made by one pass over the line graph (k_row_classes),
 // and a closed instance takes off a term for each of its three centres.
 // Bound by instructions, 50 to 80 per 32 entries (100,000 Zipf hyperedges,
 // 200,000 draws of A+: 13.4 ms against 59.4 for the merge, whose searches by
-// shuffles go over both rows; 30,011 hyperedges, 500 samples of A: 21.4 against
-// 141.8).
+// shuffles go over both rows; 30,011 hyperedges, 500 samples of A: 24.3 against
+// 140.7).
 // ---------------------------------------------------------------------------
 constexpr int kRowsThreads = 256;
 constexpr int kRowsWarps = kRowsThreads / 32;
@@ -203,7 +203,7 @@ struct RowsArgs {
   const uint32_t* row;        // A+: staged row of the draws, grouped
   const uint32_t* draw;       //     and which draw it is (null: the draw of that place)
   const uint2* other;         //     streamed row of each draw: id and size, omega
-  const uint32_t* classes;    // A: class histograms of all rows, or null
+  const uint32_t* classes;    // A: class histograms of all rows
   int n_classes;              //    [largest size][theta + 2] each
   unsigned long long* queue;
 };

@@ -1971,7 +1971,7 @@ bool levels_kept(const mochy_ctx* ctx) { return ctx->levels && ctx->levels->read
 
 bool levels_cover(int theta, int64_t n_edges, int n_units) {
   // a tuple key has 19 bits left for the unit
-  return theta <= kMaxTheta && n_edges > 0 && n_units < (1 << 18);
+  return theta >= 1 && theta <= kMaxTheta && n_edges > 0 && n_units < (1 << 18);
 }
 
 double levels_unit_us(double entries, double n_edges) {

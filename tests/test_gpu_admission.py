@@ -88,3 +88,12 @@ def test_waves_of_a_batch_leave_room_for_the_levels():
     assert got[7]["n_waves"] > 1 and got[7]["dense_threshold"] == 0
     for a, b in zip(got[:7], ref[:7]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("theta", [0, -7])
+def test_a_bad_theta_is_refused_as_ever(theta):
+    cfg = B.mochy_config_default()
+    cfg.theta = theta
+    with pytest.raises(B.MochyError) as e:
+        B.mochy_profile_batch([_communities(1000, 3)], 1, [1], cfg)
+    assert e.value.code == B.E_INVALID

@@ -390,7 +390,8 @@ GraphBytes estimate_graph_bytes(int64_t n_nodes, int64_t n_edges, const int64_t*
                                     pairs, hubs);
     // line degrees of 2 w / E on average
     r.levels = levels_unit_us((double)level_entries((int)most, theta), (double)n_edges) <=
-               split_unit_us((double)n_edges, 4.0 * w * w / (double)n_edges);
+               split_unit_us((double)n_edges, 4.0 * w * w / (double)n_edges,
+                             std::min(w, 0.5 * (double)n_edges * (double)n_edges));
   }
   return r;
 }

@@ -288,7 +288,7 @@ int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const 
 void release_levels(mochy_ctx* ctx);                                  // levels.cu
 bool levels_kept(const mochy_ctx* ctx);                               // levels.cu
 double levels_unit_us(double entries, double n_edges);                // levels.cu
-double split_unit_us(double n_edges, double deg2);                    // levels.cu
+double split_unit_us(double n_edges, double deg2, double wedges);     // levels.cu
 int64_t level_entries(int max_size, int theta);                       // levels.cu
 double levels_bytes(double n_nodes, double n_edges, double n_inc, int max_size, int theta,
                     double wedges, double node_pairs, double hubs);   // levels.cu

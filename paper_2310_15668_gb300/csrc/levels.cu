@@ -1978,8 +1978,9 @@ double levels_unit_us(double entries, double n_edges) {
   return 9.3e-5 * pow(entries * n_edges, 0.65);
 }
 
-double split_unit_us(double n_edges, double deg2) {
-  return 0.015 * n_edges + 1.2e-5 * std::min(deg2, 2e4 * n_edges);
+double split_unit_us(double n_edges, double deg2, double wedges) {
+  const double words = wedges * n_edges / 32.0;
+  return 0.015 * n_edges + std::min(1.2e-5 * deg2, 0.24 * n_edges + 2.5e-6 * words);
 }
 
 int64_t level_entries(int max_size, int theta) {
@@ -2062,10 +2063,12 @@ static size_t triples_smem(int theta) {
 //     to 60: 0.91 against 0.42; 300 Zipf ones, theta = 4: 0.68 against 0.58, and
 //     below 512 the levels are taken as they are (launches are most of both).
 //     In a batch a unit takes 9.3e-5 (entries x hyperedges)^0.65 against 0.015 a
-//     hyperedge and 1.2e-5 a squared line degree (up to 20,000 a hyperedge, from
-//     where dense rows pay), us: units of 60 hyperedges of up to 25, 6.7 against
-//     4.0 a unit, of 250 uniform ones 20 against 14, of 250 Zipf ones 19 against
-//     30, of 2,000 Zipf ones 111 against 481.
+//     hyperedge and 1.2e-5 a squared line degree (from 20,000 a hyperedge on,
+//     where dense rows pay, that much and the words of these), us: units of 60
+//     hyperedges of up to 25, 6.7 against 4.0 a unit, of 250 uniform ones 20
+//     against 14, of 250 Zipf ones 19 against 30, of 2,000 Zipf ones 111 against
+//     481, of 2,000 to 20,000 1,800 against 14,800.  The light nodes' share is in
+//     it, unless a unit's own matrix is past the caches.
 //   * the scan, thresholds to 4 (levels against scan): 250,000 hyperedges in
 //     communities of 200 88 against 33, of 50 20 against 12; 6,000 uniform ones
 //     of up to 60 4.0 against 1.0; 4,001 Zipf ones 1.3 against 28.
@@ -2076,7 +2079,7 @@ static int levels_pay(mochy_ctx* ctx, int theta, LevelsAgainst against, const Wo
   *pay = true;
   if (lone && ctx->n_edges < 512 && against == LevelsAgainst::kSplit) return MOCHY_OK;
   const double f = (double)n_dense / E;
-  const bool far = mat_bytes >= ((size_t)256 << 20);
+  const bool far = mat_bytes / (size_t)ctx->n_units >= ((size_t)256 << 20);
   double levels = 150.0 + 0.2e-6 * (double)mat_bytes;
   if (lone || far)   // else in what a unit takes
     levels += 1e-6 * 1024.0 * ((double)w.light_pairs * (7.0 + (far ? 20.0 * f * f : 0.0)) +
@@ -2087,7 +2090,7 @@ static int levels_pay(mochy_ctx* ctx, int theta, LevelsAgainst against, const Wo
     return MOCHY_OK;
   }
   *pay = levels <= (lone ? 1.3 * (340.0 + 0.01 * E + 5e-6 * deg2)
-                         : 340.0 + split_unit_us(E, deg2));
+                         : 340.0 + U * split_unit_us(E / U, deg2 / U, (double)ctx->n_wedges / U));
   if (*pay || !lone) return MOCHY_OK;
   double sparse = 0.0, words = 0.0;
   const int rc = model_split_work(ctx, &sparse, &words);

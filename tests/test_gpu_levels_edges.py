@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_2310_15668_gb300 import binding as B
+from paper_2310_15668_gb300 import binding as B, synth
 from . import _util
 
 pytestmark = pytest.mark.gpu
@@ -248,3 +248,19 @@ def test_rows_of_16_and_17_heavy_pairs_in_a_batch():
     for g, (n, off, nodes) in enumerate(gs):
         o = oracle.profile(n, off, nodes, 1, seeds[g])
         assert np.array_equal(ch[g], o["counts_h"]) and np.array_equal(c3[g], o["counts_3h"])
+
+
+def test_batches_of_ordinary_hypergraphs_go_by_levels():
+    """Overlap matrices of 70 MB an input, more than 256 MB together: each fits the
+    caches."""
+    gs = []
+    for q in range(4):
+        spec = synth.HypergraphSpec(6000, 12000, 2, 25, "powerlaw", 2.5, "zipf", 1.0, seed=800 + q)
+        gs.append((6000, *synth.generate(spec)))
+    seeds = [1, 2, 3, 4]
+    cfg = B.mochy_config_default()
+    cfg.rest_path = 2                    # the split kernels
+    got = B.mochy_profile_batch(gs, 3, seeds)
+    ref = B.mochy_profile_batch(gs, 3, seeds, cfg)
+    assert got[7]["dense_threshold"] == 0
+    assert np.array_equal(got[4], ref[4]) and np.array_equal(got[5], ref[5])

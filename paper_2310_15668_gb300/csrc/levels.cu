@@ -204,8 +204,10 @@ __host__ __device__ inline int trip_class(int A, int theta) {
 
 // What the ways of counting have to go over (see levels_pay): the sum of the
 // squared line degrees, and what light nodes cost the levels, in units of 1,024.
+// overlaps: the overlaps of all pairs of hyperedges together (to see how large
+// they are on average).
 struct Work {
-  unsigned long long deg2, light_pairs, light_rows;
+  unsigned long long deg2, light_pairs, light_rows, overlaps;
 };
 
 // adds up n, one value a thread, over a block of kRowThreads
@@ -245,7 +247,7 @@ k_lv_rows(int64_t n_edges, const int64_t* __restrict__ noff, const int32_t* __re
 // kFewHeavy: d d' summed over the nodes d' that it shares a hyperedge with (as
 // if they were alike), and d / 2 for each of the heavy pairs.
 struct LightWork {
-  unsigned long long pairs = 0ull, rows = 0ull;
+  unsigned long long pairs = 0ull, rows = 0ull, overlaps = 0ull;
   __device__ __forceinline__ void add(int64_t d, int64_t others, int64_t many) {
     pairs += ((unsigned long long)d * d * (others + d) / 2 + 512) >> 10;
     rows += ((unsigned long long)d * many / 2 + 512) >> 10;
@@ -289,10 +291,12 @@ k_lv_nodes(LevelArgs g, int hub_deg, const int32_t* __restrict__ heavy,
       seg_b[v] = hub ? 1 : 0;
       seg_n[v] = others;
       if (!hub) light.add(e - b, others, many);
+      light.overlaps += (unsigned long long)(e - b) * (unsigned long long)(e - b - 1) / 2;
     }
   }
   block_add(light.pairs, &work->light_pairs);
   block_add(light.rows, &work->light_rows);
+  block_add(light.overlaps, &work->overlaps);
 }
 
 // Units of more hubs than kMaxHubs keep those of highest degree, the lower id
@@ -362,6 +366,7 @@ __global__ void k_lv_totals(LevelArgs g, const int64_t* __restrict__ S, int64_t 
     w[0] = (int64_t)work->deg2;
     w[1] = (int64_t)work->light_pairs;
     w[2] = (int64_t)work->light_rows;
+    w[3] = (int64_t)work->overlaps;
   }
   if (u > g.n_units) return;
   const int64_t e = g.n_units > 1 ? g.eseg[u] : (u ? g.n_edges : 0);
@@ -1851,7 +1856,8 @@ __device__ __forceinline__ Part entry_part(const LevelArgs& g, int64_t at, int p
 // The blocks go over the units (of one histogram each) and, within a unit, over
 // the chunks of its tables, all along grid.x: grid.y ends at 65,535, and a batch
 // may have more units.  The hash of tuples outside the table is one for all
-// units and is gone over once: its tuples are added to the block's histogram
+// units and is gone over once, by all blocks (there are as many as it has groups
+// of slots, up to eight an SM, if the tables have fewer chunks): its tuples are added to the block's histogram
 // when there is one unit, else to their units' in global memory.
 __global__ void __launch_bounds__(kFinishThreads)
 k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, int n_bins,
@@ -1859,13 +1865,13 @@ k_lv_finish(LevelArgs g, Coder cd, unsigned long long* __restrict__ hist_out, in
   extern __shared__ unsigned long long hists[];   // [copies][n_bins + 1]
   __shared__ int32_t queue[kFinishChunk];
   __shared__ int32_t n_queue;
-  const int unit = (int)blockIdx.x / n_chunks;
+  const int unit = min((int)blockIdx.x / n_chunks, g.n_units - 1);
   unsigned long long* hist = hists + (threadIdx.x & (copies - 1)) * (n_bins + 1);
   for (int q = threadIdx.x; q < copies * (n_bins + 1); q += kFinishThreads) hists[q] = 0ull;
   if (threadIdx.x == 0) n_queue = 0;
   __syncthreads();
   const int64_t* tab = g.tab + unit * g.tab_stride;
-  const int64_t first = (int64_t)(blockIdx.x - unit * n_chunks) * chunk;
+  const int64_t first = (int64_t)((int)blockIdx.x - unit * n_chunks) * chunk;   // past the end: none
   for (int q = threadIdx.x; q < chunk && first + q < g.n_tab; q += kFinishThreads)
     if (tab[first + q]) queue[atomicAdd(&n_queue, 1)] = q;
   __syncthreads();
@@ -1998,7 +2004,7 @@ double levels_bytes(double n_nodes, double n_edges, double n_inc, int max_size, 
   const double scan = 8.0 * (3.0 * n_edges + 2.0 * n_nodes + 4.0);
   hubs = std::min(hubs, (double)kMaxHubs);
   return 2.25 * scan + (4.0 * Q + 44.0) * n_nodes + (12.0 + 4.0 * trip_classes(theta)) * n_edges +
-         2.0 * n_inc + 16.0 * heavy + 16.0 * node_pairs + n_edges * (n_edges + 8.0) / 2.0 +
+         2.0 * n_inc + 8.0 * heavy + std::min(32.0 * heavy, 16777216.0) + 16.0 * node_pairs + n_edges * (n_edges + 8.0) / 2.0 +
          4.0 * (node_pairs + 16.0) * (8.0 + 4.0 * CP) + 4.0 * CP * hubs * hubs +
          8.0 * (double)level_entries(max_size, theta) + 65536.0;
 }
@@ -2136,7 +2142,7 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against)
   const size_t b_scan = al((size_t)(n_seg + 1) * 8), b_ncls = al((size_t)N * Q * 4),
                b_hplus = al((size_t)E * 4), b_ehub = al((size_t)T * 2),
                b_unit = al((size_t)U * sizeof(LevelUnit)),
-               b_tot = al((size_t)(3 + 2 * (U + 1) + 3) * 8);
+               b_tot = al((size_t)(3 + 2 * (U + 1) + 4) * 8);
   lv->bytes[0] = b_scan + b_ncls + 2 * b_hplus + b_ehub + b_unit + b_tot;
   if (!room_for(ctx, lv->bytes[0] + scratch_growth(ctx, 0, (size_t)(n_seg + 1) * 8 + sizeof(Work))))
     return fail(MOCHY_E_NOMEM, "level structures past the reserved memory");
@@ -2161,7 +2167,7 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against)
   k_lv_nodes<<<row_grid(ctx, N, 8), kRowThreads, 0, st>>>(g, kHubDeg, ctx->heavy_deg, ncls, seg + o_b,
                                                          seg + o_n, d_work);
   MOCHY_LAUNCHED();
-  std::vector<int64_t> tot((size_t)3 + 2 * (U + 1) + 3);
+  std::vector<int64_t> tot((size_t)3 + 2 * (U + 1) + 4);
   const int64_t* hub_tot = tot.data() + 3 + U + 1;   // first hub of each unit
   for (bool ranked = false;; ranked = true) {
     MOCHY_TRY(scan_exclusive_i64(ctx, seg, scan, n_seg + 1));
@@ -2226,9 +2232,10 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against)
   g.o_trip = g.o_out2 + n2;
   g.n_tab = g.o_trip + g.tt.total;
   g.tab_stride = (g.n_tab + 31) & ~(int64_t)31;
+  const int64_t* tw = tot.data() + 3 + 2 * (U + 1);
+  const Work w{(unsigned long long)tw[0], (unsigned long long)tw[1], (unsigned long long)tw[2],
+               (unsigned long long)tw[3]};
   if (against != LevelsAgainst::kNothing) {
-    const int64_t* tw = tot.data() + 3 + 2 * (U + 1);
-    const Work w{(unsigned long long)tw[0], (unsigned long long)tw[1], (unsigned long long)tw[2]};
     bool pay;
     MOCHY_TRY(levels_pay(ctx, theta, against, w, g.n_tab, (size_t)mwords * 4, tot[3 + U], &pay));
     if (!pay) {
@@ -2240,8 +2247,15 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against)
                              cudaMemcpyHostToDevice, st));
   uint64_t slots = 64;
   while (slots < (uint64_t)(2 * P)) slots <<= 1;
+  // The hash of tuples outside the table.  A tuple that finds no slot costs 256
+  // probes and some 60 global atomics, so it is sized for the distinct ones: up
+  // to 0.07 a heavy entry where overlaps are 1.2 on average, 0.37 and 0.71 where
+  // they are 1.4 and 3.5 (700 hyperedges of 6 to 16 of 70 nodes, theta = 4: 87 ms
+  // with a quarter of a slot an entry, 3.2 with one).
+  const bool wide = (double)w.overlaps > 1.3 * (double)ctx->n_wedges;
+  const int64_t want = wide ? H : H / 4;
   uint64_t oslots = 1 << 12;
-  while (oslots < (1u << 18) && (int64_t)oslots < H / 4) oslots <<= 1;
+  while (oslots < (wide ? 1u << 20 : 1u << 18) && (int64_t)oslots < want) oslots <<= 1;
   const size_t b_hadj = al((size_t)std::max<int64_t>(H, 1) * 8),
                b_adj = al((size_t)std::max<int64_t>(NB, 1) * 8),
                b_mat = al((size_t)std::max<int64_t>(mwords, 1) * 4), b_key = al(slots * 8),
@@ -2381,7 +2395,10 @@ int launch_levels(mochy_ctx* ctx, unsigned long long* d_hist, int n_bins, const 
     chunk *= 2;
   while (copies > 1 && (size_t)copies * (n_bins + 1) * 8 > 32 * 1024) copies /= 2;
   const int n_chunks = ceil_div(g.n_tab, chunk);
-  k_lv_finish<<<(unsigned)n_chunks * (unsigned)g.n_units, kFinishThreads,
+  const unsigned n_blocks =
+      std::max((unsigned)n_chunks * (unsigned)g.n_units,
+               (unsigned)std::min<uint64_t>((g.omask + 1) / kFinishThreads, (uint64_t)ctx->num_sms * 8));
+  k_lv_finish<<<n_blocks, kFinishThreads,
                 (size_t)copies * (n_bins + 1) * 8, st>>>(g, cd, d_hist, n_bins, n_chunks, chunk,
                                                          copies);
   MOCHY_LAUNCHED();

@@ -2251,7 +2251,7 @@ static int prepare(mochy_ctx* ctx, Levels* lv, int theta, LevelsAgainst against)
   // probes and some 60 global atomics, so it is sized for the distinct ones: up
   // to 0.07 a heavy entry where overlaps are 1.2 on average, 0.37 and 0.71 where
   // they are 1.4 and 3.5 (700 hyperedges of 6 to 16 of 70 nodes, theta = 4: 87 ms
-  // with a quarter of a slot an entry, 3.2 with one).
+  // with a quarter of a slot an entry, 7.3 with one).
   const bool wide = (double)w.overlaps > 1.3 * (double)ctx->n_wedges;
   const int64_t want = wide ? H : H / 4;
   uint64_t oslots = 1 << 12;

@@ -221,7 +221,7 @@ __device__ __forceinline__ void block_add(unsigned long long n, unsigned long lo
     for (int w = 0; w < kRowWarps; ++w) s += part[w];
     if (s) atomicAdd(out, s);
   }
-  __syncthreads();
+  __syncthreads();   // the next call's sums
 }
 
 // heavy degrees, which rows can be in a triangle of heavy pairs, and node
@@ -294,9 +294,19 @@ k_lv_nodes(LevelArgs g, int hub_deg, const int32_t* __restrict__ heavy,
       light.overlaps += (unsigned long long)(e - b) * (unsigned long long)(e - b - 1) / 2;
     }
   }
-  block_add(light.pairs, &work->light_pairs);
-  block_add(light.rows, &work->light_rows);
-  block_add(light.overlaps, &work->overlaps);
+  // the sums of the warps, three neighbouring counters
+  __shared__ unsigned long long part[3][kRowWarps];
+  if (lane == 0) {
+    part[0][threadIdx.x >> 5] = light.pairs;
+    part[1][threadIdx.x >> 5] = light.rows;
+    part[2][threadIdx.x >> 5] = light.overlaps;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    unsigned long long s = 0ull;
+    for (int w = 0; w < kRowWarps; ++w) s += part[threadIdx.x][w];
+    if (s) atomicAdd(&work->light_pairs + threadIdx.x, s);
+  }
 }
 
 // Units of more hubs than kMaxHubs keep those of highest degree, the lower id
